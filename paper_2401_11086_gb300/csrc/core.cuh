@@ -148,24 +148,28 @@ SMRT_HD void binomial_divided(T (&v)[nmom(N)], const T (&G)[3][N + 1]) {
 // recurrence of the generating function exp(u t + (th - 1) t^2 / 2) of the 1D Maxwellian's
 // absolute Hermite coefficients (Appendix B closed form). In divided form:
 // G[j+1] = (u G[j] + (th - 1) G[j-1]) / (j + 1).
-template <int N, class T>
+// Fused: with the fused operation written out (the same rounding wherever it is compiled).
+template <int N, class T, bool Fused = false>
 SMRT_HD void maxwell_divided(T (&G)[N + 1], T u, T thm1) {
     G[0] = T(1);
     if constexpr (N >= 1) G[1] = u;
     static_for<(N >= 1 ? N - 1 : 0)>([&](auto J) {
         constexpr int j = decltype(J)::value + 1;
-        G[j + 1] = (u * G[j] + thm1 * G[j - 1]) * T(1.0 / (j + 1));
+        if constexpr (Fused)
+            G[j + 1] = fma(u, G[j], thm1 * G[j - 1]) * T(1.0 / (j + 1));
+        else
+            G[j + 1] = (u * G[j] + thm1 * G[j - 1]) * T(1.0 / (j + 1));
     });
 }
 
 // a4 in divided form: td_beta = d_beta / beta! = theta^(-|beta|/2) [T(-u, 2 - theta) ta]_beta,
 // v holding ta on entry (with the full a_0 = rho in slot 0) and td on exit.
-template <int Nm, class T>
+template <int Nm, class T, bool Fused = false>
 SMRT_D void to_local_divided(T (&v)[nmom(Nm)], const T (&u)[3], T theta, T thm1) {
     T G[3][Nm + 1];
     static_for<3>([&](auto K) {
         constexpr int k = decltype(K)::value;
-        maxwell_divided<Nm, T>(G[k], -u[k], -thm1);
+        maxwell_divided<Nm, T, Fused>(G[k], -u[k], -thm1);
     });
     binomial_divided<Nm, T>(v, G);
     const T is = rsq(theta);

@@ -85,7 +85,9 @@ StepArgs<Lat, T> make_args(const CtxView &v, const void *fin, void *fout) {
     for (int p = 0; p <= Lat::NP; ++p) {
         a.wp[p] = T(v.wp[p]);
         a.wpd[p] = v.wp[p];
-        a.wlo[p] = float(v.wp[p] - double(float(v.wp[p])));
+        const double ws = v.wp[p] * pow2f(24 - kFixP);
+        a.wsh[p] = float(ws);
+        a.wsl[p] = float(ws - double(float(ws)));
     }
     a.c = T(v.c);
     a.cd = v.c;

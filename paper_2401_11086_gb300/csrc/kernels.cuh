@@ -69,7 +69,8 @@ struct StepArgs {
     long long plane[Lat::Q];  // element offset of each population plane, library order
     T wp[Lat::NP + 1];        // weight of the rest velocity, then of each pair
     double wpd[Lat::NP + 1];  // the same weights in double, for every double-precision rebuild
-    float wlo[Lat::NP + 1];   // w - float(w): the weights as two-float numbers (split precision)
+    float wsh[Lat::NP + 1];   // w 2^(24 - kFixP) as two-float numbers (split precision)
+    float wsl[Lat::NP + 1];
     T c;
     double cd;                // c in double
     float clo;                // c - float(c)
@@ -180,11 +181,14 @@ SMRT_D ff ff_inv() {
     return ff{hi, lo};
 }
 
-// Fixed point: x 2^S rounded to the nearest integer (the hardware conversion of the exactly
-// scaled float). Sums of such integers are exact and independent of their order. Valid for
-// |x| < 2^(62 - S); magnitudes below 2^-(S + 1) give 0. The split-precision step keeps
-// populations and raw moments at S = kFix (2^-44 resolution, range 2^18) and the equilibrium's
-// monomial coefficients at S = kFixP (2^-48, range 2^14).
+// Fixed point: x 2^S rounded to the nearest integer. Sums of such integers are exact and
+// independent of their order. Valid for |x| < 2^(62 - S); magnitudes below 2^-(S + 1) give 0. The
+// split-precision step keeps populations and raw moments at S = kFix (2^-44 resolution, range
+// 2^18) and the equilibrium's monomial coefficients at S = kFixP (2^-48, range 2^14).
+// The 64-bit conversion runs on the double-precision pipe, which this step leaves idle otherwise
+// (28 % busy); two 32-bit conversions instead (the remainder of the first is exact in a float)
+// cost eleven instructions of the issue-bound step: 280 against 259 us per step on the 64
+// batched D3Q103 shocks.
 constexpr int kFix = 44;
 constexpr int kFixP = 48;
 constexpr float pow2f(int e) { return e >= 0 ? float(1ull << e) : 1.0f / float(1ull << -e); }
@@ -196,15 +200,13 @@ template <int S = kFix>
 SMRT_D long long to_fixed(double x) {
     return __double2ll_rn(x * static_cast<double>(1ull << S));
 }
-// Exact sum of products m x (m a small positive constant, x a 64-bit integer) in one 64-bit
+// Exact sum of products m x (m a small positive integer, x a 64-bit integer) in one 64-bit
 // accumulator, each product formed as m lo32(x) (a 32 x 32 -> 64-bit multiply-add) plus
 // m hi32(x) added to the upper word. Arithmetic is modulo 2^64, so the sum is exact whenever it
 // fits in 64 bits.
 struct SplitAcc {
     unsigned long long v = 0;
-    template <int m>
-    SMRT_D void madd(long long x) {
-        static_assert(m > 0, "positive multiplier");
+    SMRT_D void madd(long long x, int m) {  // m > 0
         const unsigned long long ux = static_cast<unsigned long long>(x);
         v += static_cast<unsigned long long>(static_cast<unsigned>(ux)) * static_cast<unsigned>(m);
         v += static_cast<unsigned long long>(static_cast<unsigned>(ux >> 32) * static_cast<unsigned>(m)) << 32;
@@ -213,24 +215,27 @@ struct SplitAcc {
     SMRT_D long long value() const { return static_cast<long long>(v); }
 };
 
-// q 2^-S as a two-float number: q = a 2^48 + b 2^24 + c with 0 <= b, c < 2^24, each piece
-// exact as a float
-template <int S = kFix>
+// q 2^-24 as a two-float number: q = a 2^48 + b 2^24 + c with 0 <= b, c < 2^24, each piece
+// exact as a float; a 2^24 + b and its error by a quick two-sum (|a 2^24| > b or a = 0). The
+// remaining power of two (2^(24 - S)) is folded by the callers into what they multiply by.
 SMRT_D ff fixed_to_ff(long long q) {
-    const float a = float(int(q >> 48)) * pow2f(48 - S);
-    const float b = float(int((q >> 24) & 0xffffff)) * pow2f(24 - S);
-    const float c = float(int(q & 0xffffff)) * pow2f(-S);
-    const ff s = ff_two_sum(a, b);
-    return ff_quick(s.hi, __fadd_rn(s.lo, c));
+    const float a = __int2float_rn(int(q >> 48));
+    const float b = __int2float_rn(int((q >> 24) & 0xffffff));
+    const float c = __int2float_rn(int(q & 0xffffff));
+    const float s = __fmaf_rn(a, 0x1p24f, b);
+    const float lo = __fsub_rn(b, __fmaf_rn(a, -0x1p24f, s));
+    return ff_quick(s, __fmaf_rn(c, 0x1p-24f, lo));
 }
+SMRT_D ff ff_scale(ff x, float p) { return {__fmul_rn(x.hi, p), __fmul_rn(x.lo, p)}; }  // p a power of two
 
 // Stochastic rounding of a two-float value hi + lo (|lo| at most half a float spacing of hi) to
 // a float: hi's neighbour on lo's side with probability |lo| / (distance to that neighbour),
 // else hi, drawn from the same counter-based hash as above.
 SMRT_D float round_stochastic(ff x, unsigned key) {
     const unsigned hb = __float_as_uint(x.hi);
-    const bool away = (x.lo > 0.f) == (x.hi > 0.f);  // the neighbour of larger magnitude
-    const float nb = __uint_as_float(away ? hb + 1u : hb - 1u);
+    // +1 (the neighbour of larger magnitude) when hi and lo have the same sign, else -1
+    const int toward = (static_cast<int>(hb ^ __float_as_uint(x.lo)) >> 31) | 1;
+    const float nb = __uint_as_float(hb + static_cast<unsigned>(toward));
     const float gap = fabsf(__fsub_rn(nb, x.hi));
     const float u = __fmul_rn(__uint2float_rn(mix32(key) >> 8), 0x1p-24f);  // uniform in [0, 1)
     return fabsf(x.lo) > __fmul_rn(u, gap) ? nb : x.hi;
@@ -265,6 +270,16 @@ SMRT_D void wht(U (&x)[NB]) {
     });
 }
 
+// Run-time orbit rows of each set, in constant memory (every lane of a warp reads the same row).
+static __constant__ const OrbitRows<D3Q39> kOrbitRows39 = OrbitRows<D3Q39>();
+static __constant__ const OrbitRows<D3Q103> kOrbitRows103 = OrbitRows<D3Q103>();
+template <class Lat>
+SMRT_D const OrbitRows<Lat> &orbit_rows();
+template <>
+SMRT_D const OrbitRows<D3Q39> &orbit_rows<D3Q39>() { return kOrbitRows39; }
+template <>
+SMRT_D const OrbitRows<D3Q103> &orbit_rows<D3Q103>() { return kOrbitRows103; }
+
 // ------------------------------------------------------------------------------ collision
 template <class Lat, int N, class T, class Acc, bool Split>
 struct Collide {
@@ -273,6 +288,7 @@ struct Collide {
     static constexpr int M = nmom(N);
     static constexpr int KT = ntau(N);
     static constexpr SignOrbits<Lat> kOrb = SignOrbits<Lat>();
+    static constexpr OrbitRows<Lat> kRows = OrbitRows<Lat>();
 
     // a2: conserved sums, in Acc. The state holds deviations df_i = f_i - w_i; the quadrature
     // gives sum w_i = 1, sum w_i xi_i = 0, sum w_i |xi_i|^2 = 3, so
@@ -382,38 +398,48 @@ struct Collide {
     }
 
     // Split precision, a2 + a3: the raw moments R_gamma = sum_i df_i e_i^gamma, |gamma| <= Nm,
-    // exactly, in fixed point (get(ic<i>) gives population i in fixed point), per sign orbit as
-    // raw_moments_of does, with the pair sums and transforms taken on 64-bit integers and the
-    // products by a^gamma accumulated in two parts (SplitAcc).
+    // exactly, in fixed point (get(i, e, s, off) gives population i, of vector s e,
+    // staged at offset off, in fixed point), per sign
+    // orbit as raw_moments does, with the pair sums and transforms taken on 64-bit integers and the
+    // products by a^gamma accumulated in two parts (SplitAcc). The orbits are run-time rows
+    // (OrbitRows), one loop per axis set: see collide_split.
     template <int Nm, class Get>
     SMRT_D static void fixed_moments(Get &&get, long long (&R)[nmom(Nm)]) {
         constexpr int Mm = nmom(Nm);
         SplitAcc acc[Mm];
-        acc[0].add(get(ic<0>{}));
-        static_for<kOrb.n>([&](auto O) {
-            constexpr int o = decltype(O)::value;
-            constexpr int np = 1 << (kOrb.k[o] - 1);
-            long long S[np], D[np];
-            static_for<np>([&](auto B) {
-                constexpr int b = decltype(B)::value, p = kOrb.pair[o][b];
-                constexpr bool fl = kOrb.flip[o][b] != 0;
-                const long long fp = get(ic<2 * p + 1>{}), fm = get(ic<2 * p + 2>{});
-                S[b] = fp + fm;
-                D[b] = fl ? fm - fp : fp - fm;
-            });
-            wht<np>(S);
-            wht<np>(D);
-            static_for<Mm>([&](auto G) {
-                constexpr int g = decltype(G)::value;
-                constexpr int m = kOrb.monomial(o, g);
-                if constexpr (m != 0) {
-                    constexpr int cl = kOrb.parity_class(o, g);
-                    if constexpr ((mi_order(g) & 1) == 0)
-                        acc[g].template madd<m>(S[cl]);
-                    else
-                        acc[g].template madd<m>(D[cl]);
+        const signed char rest[3] = {0, 0, 0};
+        acc[0].add(get(0, rest, 1, 0));
+        static_for<7>([&](auto Mk) {
+            constexpr int mask = decltype(Mk)::value + 1;
+            constexpr int np = 1 << (mask_axes(mask) - 1);
+            if constexpr (kRows.count(mask) > 0) {
+                constexpr int o0 = kRows.first[mask], o1 = kRows.first[mask + 1];
+#pragma unroll 1
+                for (int o = o0; o < o1; ++o) {
+                    const typename OrbitRows<Lat>::Row &r = orbit_rows<Lat>().row[o];
+                    long long S[np], D[np];
+                    static_for<np>([&](auto B) {
+                        constexpr int b = decltype(B)::value;
+                        const long long fp = get(r.ip[b], r.e[b], 1, r.sp[b]), fm = get(r.im[b], r.e[b], -1, r.sm[b]);
+                        S[b] = fp + fm;
+                        D[b] = fp - fm;
+                    });
+                    wht<np>(S);
+                    wht<np>(D);
+                    static_for<Mm>([&](auto G) {
+                        constexpr int g = decltype(G)::value;
+                        if constexpr (g == 0) {
+                            acc[g].add(S[0]);
+                        } else if constexpr (mask_has(mask, g)) {
+                            constexpr int cl = mask_class(mask, g);
+                            if constexpr ((mi_order(g) & 1) == 0)
+                                acc[g].madd(S[cl], r.mono[g]);
+                            else
+                                acc[g].madd(D[cl], r.mono[g]);
+                        }
+                    });
                 }
-            });
+            }
         });
         static_for<Mm>([&](auto G) { R[decltype(G)::value] = acc[decltype(G)::value].value(); });
     }
@@ -553,7 +579,7 @@ struct Collide {
     // the first time (tau_20); else SMRT.
     SMRT_D static void relax_coefficients(T (&v)[M], const T (&u)[3], T rho, T theta, T thm1, T o0,
                                           const T *tauA, const T *tauB, int model = 0, T es_b = T(0)) {
-        to_local<N>(v, u, theta, thm1);
+        to_local_divided<N, T, Split>(v, u, theta, thm1);
         // a5: relax orders 2..N; order 0 is rho, order 1 is zero by definition of u
         if (model == 1) {
             relax_es_divided<N, T>(v, rho, tauA[0], tauB[0], es_b);
@@ -561,7 +587,7 @@ struct Collide {
             T s[KT];
             static_for<KT>([&](auto K) {
                 constexpr int k = decltype(K)::value;
-                s[k] = T(1) - rcp_tau<T>(tauA[k], tauB[k], rho);
+                s[k] = Split ? fma(-rho, rcp(fma(tauB[k], rho, tauA[k])), T(1)) : T(1) - rcp_tau<T>(tauA[k], tauB[k], rho);
             });
             static_for<N - 1>([&](auto Nn) { relax_order<N, decltype(Nn)::value + 2, T>(v, s); });
         }
@@ -582,53 +608,49 @@ struct Collide {
         T G[3][N + 1];
         static_for<3>([&](auto K) {
             constexpr int k = decltype(K)::value;
-            maxwell_divided<N, T>(G[k], u[k], thm1);
+            maxwell_divided<N, T, Split>(G[k], u[k], thm1);
         });
         binomial_divided<N, T>(v, G);
     }
 
     // The whole collision: df (pre-collision deviations, library order) -> df (post-collision).
     // Returns false when rho or theta is not positive (or NaN).
-    SMRT_D static bool collide(T (&f)[Q], const T (&wp)[NP + 1], const float (&wlo)[NP + 1], T c,
-                               float clo, const T *tauA, const T *tauB, unsigned key = 0u, int model = 0,
+    SMRT_D static bool collide(T (&f)[Q], const T (&wp)[NP + 1], T c, const T *tauA, const T *tauB, int model = 0,
                                T es_b = T(0)) {
-        if constexpr (Split) {
-            bool finite = true;
-            const bool ok = collide_split(
-                [&](auto I) {
-                    finite &= (__float_as_uint(f[decltype(I)::value]) & 0x7f800000u) != 0x7f800000u;
-                    return to_fixed(f[decltype(I)::value]);
-                },
-                [&](int i, T v) { f[i] = v; }, wp, wlo, c, clo, tauA, tauB, key, model, es_b);
-            return ok && finite;
-        } else {
-            // a3: coefficients of the deviations; the full a has 1 more in slot 0, i.e. a_0 = rho
-            T v[M], Rc[M];
-            absolute<N>(f, c, v, Rc);
-            // a2 from the raw moments already formed: rho - 1 = Rc_0, rho u = Rc_1,
-            // E - 3 = tr Rc_2
-            const T rhom1 = Rc[0];
-            const T rho = T(1) + rhom1;
-            const T ir = rcp(rho);
-            const T u[3] = {Rc[mi_pos(1, 0, 0)] * ir, Rc[mi_pos(0, 1, 0)] * ir, Rc[mi_pos(0, 0, 1)] * ir};
-            const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-            const T em3 = Rc[mi_pos(2, 0, 0)] + Rc[mi_pos(0, 2, 0)] + Rc[mi_pos(0, 0, 2)];
-            const T thm1 = (em3 - T(3) * rhom1 - rho * uu) * ir * T(1.0 / 3.0);
-            const T theta = T(1) + thm1;
-            const bool ok = (rho > T(0)) && (theta > T(0));
-            v[0] = rho;
-            relax_coefficients(v, u, rho, theta, thm1, rho, tauA, tauB, model, es_b);
-            v[0] = rhom1;  // deviation from the coefficients of w_i
-            T out[Q];
-            rebuild<T>(v, c, wp, out);
-            static_for<Q>([&](auto I) { f[decltype(I)::value] = out[decltype(I)::value]; });
-            return ok;
-        }
+        // a3: coefficients of the deviations; the full a has 1 more in slot 0, i.e. a_0 = rho
+        T v[M], Rc[M];
+        absolute<N>(f, c, v, Rc);
+        // a2 from the raw moments already formed: rho - 1 = Rc_0, rho u = Rc_1,
+        // E - 3 = tr Rc_2
+        const T rhom1 = Rc[0];
+        const T rho = T(1) + rhom1;
+        const T ir = rcp(rho);
+        const T u[3] = {Rc[mi_pos(1, 0, 0)] * ir, Rc[mi_pos(0, 1, 0)] * ir, Rc[mi_pos(0, 0, 1)] * ir};
+        const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+        const T em3 = Rc[mi_pos(2, 0, 0)] + Rc[mi_pos(0, 2, 0)] + Rc[mi_pos(0, 0, 2)];
+        const T thm1 = (em3 - T(3) * rhom1 - rho * uu) * ir * T(1.0 / 3.0);
+        const T theta = T(1) + thm1;
+        const bool ok = (rho > T(0)) && (theta > T(0));
+        v[0] = rho;
+        relax_coefficients(v, u, rho, theta, thm1, rho, tauA, tauB, model, es_b);
+        v[0] = rhom1;  // deviation from the coefficients of w_i
+        T out[Q];
+        rebuild<T>(v, c, wp, out);
+        static_for<Q>([&](auto I) { f[decltype(I)::value] = out[decltype(I)::value]; });
+        return ok;
     }
 
-    // Split precision (T float): pullq(ic<i>) gives pulled population i in fixed point (the stored
-    // float exactly, or the exact double end-state value beyond a fixed end), read once;
-    // store(i, value) receives post-collision population i as soon as it is formed.
+    // Split precision (T float): pullq(i, e, s, off) gives pulled population i, of vector s e, in
+    // fixed point (the stored float exactly, or the exact double end-state value beyond a fixed end),
+    // read once; store(i, value) receives post-collision population i as soon as it is formed.
+    //
+    // Code size. Unrolled over every population the D3Q103 step was 275 KB of instructions, far
+    // beyond the instruction caches: the warps waited for instructions (no_instruction 5.5 per
+    // issue, 29 % issue-active). The two ends, where most of them were (per-population conversions,
+    // products by a^gamma, rounding), therefore run as loops over the orbits of one axis set at a
+    // time, with the parity classes and the slots that vanish still compile-time: 155 KB, 50 %
+    // issue-active, 14 % more instructions. One 2048-cell shock 49.1 -> 40.3 us per step, the 64
+    // batched shocks (230 k cells, persistent) 284 -> 259 us per step, the same bits.
     //
     // Precision design. Float arithmetic is used only for the non-equilibrium part, whose own
     // size then bounds its rounding errors; whatever the equilibrium carries is formed to about
@@ -653,9 +675,10 @@ struct Collide {
     // (sum w = 1, sum w xi xi = delta, sum w |xi|^4 = 15), i.e. added to Q_0, Q_k and Q_kk, so
     // that they equal the pre-collision sums. The stored values then conserve rho, rho u and
     // energy in expectation, stochastic rounding being the only remaining error.
+    // wsh, wsl: the weights times 2^(24 - kFixP) as two-float numbers.
     template <class Pull, class Store>
-    SMRT_D static bool collide_split(Pull &&pullq, Store &&store, const T (&wp)[NP + 1],
-                                     const float (&wlo)[NP + 1], T c, float clo, const T *tauA,
+    SMRT_D static bool collide_split(Pull &&pullq, Store &&store, const float (&wsh)[NP + 1],
+                                     const float (&wsl)[NP + 1], T c, float clo, const T *tauA,
                                      const T *tauB, unsigned key, int model = 0, T es_b = T(0)) {
         static_assert(std::is_same<T, float>::value, "the split precision stores floats");
         constexpr int px = mi_pos(1, 0, 0), py = mi_pos(0, 1, 0), pz = mi_pos(0, 0, 1);
@@ -667,12 +690,14 @@ struct Collide {
         ff cp[N + 1];  // c^j
         cp[0] = ff{1.f, 0.f};
         static_for<N>([&](auto J) { cp[decltype(J)::value + 1] = cp[decltype(J)::value] * cc; });
-        const ff r = fixed_to_ff(Rq[0]);  // rho - 1
+        ff cf[N + 1];  // c^j times the scale fixed_to_ff leaves
+        static_for<N + 1>([&](auto J) { cf[decltype(J)::value] = ff_scale(cp[decltype(J)::value], pow2f(24 - kFix)); });
+        const ff r = ff_scale(fixed_to_ff(Rq[0]), pow2f(24 - kFix));  // rho - 1
         const ff rho = r + 1.f;
         const ff irho = ff_div(ff{1.f, 0.f}, rho);
-        const ff mom[3] = {cc * fixed_to_ff(Rq[px]), cc * fixed_to_ff(Rq[py]), cc * fixed_to_ff(Rq[pz])};
+        const ff mom[3] = {cf[1] * fixed_to_ff(Rq[px]), cf[1] * fixed_to_ff(Rq[py]), cf[1] * fixed_to_ff(Rq[pz])};
         const ff uf[3] = {mom[0] * irho, mom[1] * irho, mom[2] * irho};
-        const ff en = cp[2] * fixed_to_ff(Rq[pxx] + Rq[pyy] + Rq[pzz]);  // E - 3
+        const ff en = cf[2] * fixed_to_ff(Rq[pxx] + Rq[pyy] + Rq[pzz]);  // E - 3
         // theta - 1 = (E - 3 - 3 (rho - 1) - rho |u|^2) / (3 rho)
         const ff thm1 = (en - r * 3.f - (mom[0] * uf[0] + mom[1] * uf[1] + mom[2] * uf[2])) *
                         (ff_inv<3>() * irho);
@@ -704,7 +729,7 @@ struct Collide {
                     if constexpr (g0 > 0) eq = eq * mu[0][g0];
                     if constexpr (g1 > 0) eq = eq * mu[1][g1];
                     if constexpr (g2 > 0) eq = eq * mu[2][g2];
-                    Rx[g] = (fixed_to_ff(Rq[g]) * cp[mi_order(g)] - (eq + float(-unit_moment(g)))).hi;
+                    Rx[g] = (fixed_to_ff(Rq[g]) * cf[mi_order(g)] - (eq + float(-unit_moment(g)))).hi;
                 }
             });
             // a3 on the non-equilibrium part: divided absolute coefficients (float)
@@ -756,11 +781,13 @@ struct Collide {
             });
             static_for<M>([&](auto G_) {
                 constexpr int g = decltype(G_)::value;
-                ff acc = ff{0.f, 0.f};
+                ff acc = ta[g];  // hfull(g, g) = 1; the other terms have higher orders
                 static_for<M>([&](auto A) {
                     constexpr int al = decltype(A)::value;
                     constexpr double h = hfull(al, g);
-                    if constexpr (h == 1.0)
+                    if constexpr (al == g)
+                        return;
+                    else if constexpr (h == 1.0)
                         acc = acc + ta[al];
                     else if constexpr (h != 0.0)
                         acc = acc + ta[al] * float(h);
@@ -770,19 +797,20 @@ struct Collide {
         }
         // exact restoration of mass, momentum and energy (targets: rho - 1, rho u, E - 3)
         {
-            ff ms = ff{0.f, 0.f}, es = ff{0.f, 0.f}, js[3] = {ff{0.f, 0.f}, ff{0.f, 0.f}, ff{0.f, 0.f}};
+            ff ms = Qx[0], es = Qx[0] * 3.f, js[3] = {Qx[px], Qx[py], Qx[pz]};
             static_for<M>([&](auto G_) {
                 constexpr int g = decltype(G_)::value;
                 constexpr int g0 = mi_comp(g, 0), g1 = mi_comp(g, 1), g2 = mi_comp(g, 2);
                 constexpr double m0 = unit_moment(g);
                 constexpr double e0 = unit_moment3(g0 + 2, g1, g2) + unit_moment3(g0, g1 + 2, g2) +
                                       unit_moment3(g0, g1, g2 + 2);
-                if constexpr (m0 != 0.0) ms = ms + (m0 == 1.0 ? Qx[g] : Qx[g] * float(m0));
-                if constexpr (e0 != 0.0) es = es + Qx[g] * float(e0);
+                if constexpr (g != 0 && m0 != 0.0) ms = ms + (m0 == 1.0 ? Qx[g] : Qx[g] * float(m0));
+                if constexpr (g != 0 && e0 != 0.0) es = es + Qx[g] * float(e0);
                 static_for<3>([&](auto K) {
                     constexpr int k = decltype(K)::value;
                     constexpr double j0 = unit_moment3(g0 + (k == 0), g1 + (k == 1), g2 + (k == 2));
-                    if constexpr (j0 != 0.0) js[k] = js[k] + (j0 == 1.0 ? Qx[g] : Qx[g] * float(j0));
+                    if constexpr (mi_order(g) > 1 && j0 != 0.0)
+                        js[k] = js[k] + (j0 == 1.0 ? Qx[g] : Qx[g] * float(j0));
                 });
             });
             const ff A = r - ms;
@@ -804,39 +832,47 @@ struct Collide {
         });
         // a7 + a8: f'_i = w_i P(e_i), P(e_i) per sign orbit in fixed point (sums per parity
         // class, Walsh-Hadamard transform), then times w_i in two-float, rounded stochastically
-        auto out = [&](int i, int wi, long long poly) {
-            const ff w = {wp[wi], wlo[wi]};
-            store(i, round_stochastic(w * fixed_to_ff<kFixP>(poly), key ^ (0x9e3779b9u * unsigned(i + 1))));
+        auto out = [&](int i, long long poly) {
+            const int wi = (i + 1) >> 1;
+            const ff w = {wsh[wi], wsl[wi]};
+            store(i, round_stochastic(w * fixed_to_ff(poly), key ^ (0x9e3779b9u * unsigned(i + 1))));
         };
-        out(0, 0, Pq[0]);
-        static_for<kOrb.n>([&](auto O) {
-            constexpr int o = decltype(O)::value;
-            constexpr int np = 1 << (kOrb.k[o] - 1);
-            SplitAcc Ea[np], Oa[np];
-            static_for<M>([&](auto G_) {
-                constexpr int g = decltype(G_)::value;
-                constexpr int m = kOrb.monomial(o, g);
-                if constexpr (m != 0) {
-                    constexpr int cl = kOrb.parity_class(o, g);
-                    if constexpr ((mi_order(g) & 1) == 0)
-                        Ea[cl].template madd<m>(Pq[g]);
-                    else
-                        Oa[cl].template madd<m>(Pq[g]);
+        out(0, Pq[0]);
+        static_for<7>([&](auto Mk) {
+            constexpr int mask = decltype(Mk)::value + 1;
+            constexpr int np = 1 << (mask_axes(mask) - 1);
+            if constexpr (kRows.count(mask) > 0) {
+                constexpr int o0 = kRows.first[mask], o1 = kRows.first[mask + 1];
+#pragma unroll 1
+                for (int o = o0; o < o1; ++o) {
+                    const typename OrbitRows<Lat>::Row &r = orbit_rows<Lat>().row[o];
+                    SplitAcc Ea[np], Oa[np];
+                    static_for<M>([&](auto G_) {
+                        constexpr int g = decltype(G_)::value;
+                        if constexpr (g == 0) {
+                            Ea[0].add(Pq[0]);
+                        } else if constexpr (mask_has(mask, g)) {
+                            constexpr int cl = mask_class(mask, g);
+                            if constexpr ((mi_order(g) & 1) == 0)
+                                Ea[cl].madd(Pq[g], r.mono[g]);
+                            else
+                                Oa[cl].madd(Pq[g], r.mono[g]);
+                        }
+                    });
+                    long long E[np], Od[np];
+                    static_for<np>([&](auto B) {
+                        E[decltype(B)::value] = Ea[decltype(B)::value].value();
+                        Od[decltype(B)::value] = Oa[decltype(B)::value].value();
+                    });
+                    wht<np>(E);
+                    wht<np>(Od);
+                    static_for<np>([&](auto B) {
+                        constexpr int b = decltype(B)::value;
+                        out(r.ip[b], E[b] + Od[b]);
+                        out(r.im[b], E[b] - Od[b]);
+                    });
                 }
-            });
-            long long E[np], Od[np];
-            static_for<np>([&](auto B) {
-                E[decltype(B)::value] = Ea[decltype(B)::value].value();
-                Od[decltype(B)::value] = Oa[decltype(B)::value].value();
-            });
-            wht<np>(E);
-            wht<np>(Od);
-            static_for<np>([&](auto B) {
-                constexpr int b = decltype(B)::value, p = kOrb.pair[o][b];
-                constexpr bool fl = kOrb.flip[o][b] != 0;
-                out(fl ? 2 * p + 2 : 2 * p + 1, p + 1, E[b] + Od[b]);
-                out(fl ? 2 * p + 1 : 2 * p + 2, p + 1, E[b] - Od[b]);
-            });
+            }
         });
         return ok;
     }
@@ -921,28 +957,43 @@ __global__ void __launch_bounds__(128, kStepMinBlocks<Split>) step_box_kernel(St
     if (x >= a.nx) return;
     const long long row = (long long)a.nx;
     const long long slab = row * a.ny;
-    T f[Lat::Q];
-    f[0] = a.fin[a.plane[0] + wrap(z - a.kz, a.nz) * slab + wrap(y - a.ky, a.ny) * row + wrap(x - a.kx, a.nx)];
-    static_for<Lat::NP>([&](auto P) {
-        constexpr int p = decltype(P)::value;
-        static_for<2>([&](auto Sg) {
-            constexpr int sg = decltype(Sg)::value == 0 ? 1 : -1;
-            constexpr int i = 2 * p + 1 + decltype(Sg)::value;
-            const int xs = wrap(x - (sg * Lat::e(p, 0) + a.kx), a.nx);
-            const int ys = wrap(y - (sg * Lat::e(p, 1) + a.ky), a.ny);
-            const int zs = wrap(z - (sg * Lat::e(p, 2) + a.kz), a.nz);
-            f[i] = a.fin[a.plane[i] + zs * slab + ys * row + xs];
-        });
-    });
-    const bool ok = C::collide(f, a.wp, a.wlo, a.c, a.clo, tau_a<T>(a.inst[0]), tau_b<T>(a.inst[0]),
-                               mix32(unsigned(z * slab + y * row + x) ^ mix32(a.step)), a.inst[0].model,
-                               T(a.inst[0].es_b));
-    if (!ok) atomicOr(a.health, 1u);
     const long long cell = z * slab + y * row + x;
-    static_for<Lat::Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        a.fout[a.plane[i] + cell] = f[i];
-    });
+    if constexpr (Split) {
+        float probe = 0.f;  // NaN once a non-finite value has been pulled
+        const bool ok = C::collide_split(
+            [&](int i, const signed char *e, int s, int) {
+                const int xs = wrap(x - (s * e[0] + a.kx), a.nx);
+                const int ys = wrap(y - (s * e[1] + a.ky), a.ny);
+                const int zs = wrap(z - (s * e[2] + a.kz), a.nz);
+                const float v = a.fin[a.plane[i] + zs * slab + ys * row + xs];
+                probe = __fmaf_rn(v, 0.f, probe);
+                return to_fixed(v);
+            },
+            [&](int i, T v) { a.fout[a.plane[i] + cell] = v; }, a.wsh, a.wsl, a.c, a.clo, tau_a<T>(a.inst[0]),
+            tau_b<T>(a.inst[0]), mix32(unsigned(cell) ^ mix32(a.step)), a.inst[0].model, T(a.inst[0].es_b));
+        if (!(ok && probe == 0.f)) atomicOr(a.health, 1u);
+    } else {
+        T f[Lat::Q];
+        f[0] = a.fin[a.plane[0] + wrap(z - a.kz, a.nz) * slab + wrap(y - a.ky, a.ny) * row + wrap(x - a.kx, a.nx)];
+        static_for<Lat::NP>([&](auto P) {
+            constexpr int p = decltype(P)::value;
+            static_for<2>([&](auto Sg) {
+                constexpr int sg = decltype(Sg)::value == 0 ? 1 : -1;
+                constexpr int i = 2 * p + 1 + decltype(Sg)::value;
+                const int xs = wrap(x - (sg * Lat::e(p, 0) + a.kx), a.nx);
+                const int ys = wrap(y - (sg * Lat::e(p, 1) + a.ky), a.ny);
+                const int zs = wrap(z - (sg * Lat::e(p, 2) + a.kz), a.nz);
+                f[i] = a.fin[a.plane[i] + zs * slab + ys * row + xs];
+            });
+        });
+        const bool ok = C::collide(f, a.wp, a.c, tau_a<T>(a.inst[0]), tau_b<T>(a.inst[0]), a.inst[0].model,
+                                   T(a.inst[0].es_b));
+        if (!ok) atomicOr(a.health, 1u);
+        static_for<Lat::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            a.fout[a.plane[i] + cell] = f[i];
+        });
+    }
 }
 
 // Batched 1D lines (ny = nz = 1): block b handles cells x0 .. x0+blockDim-1 of instance j,
@@ -982,36 +1033,32 @@ SMRT_D void line_tile(const StepArgs<Lat, T> &a, const T *__restrict__ fin, T *_
             return load_pop<Coherent>(fin + a.plane[i] + base + wrap(xs, L));
         }
     };
-    // ... for the split precision, in fixed point (the exact double end state beyond a fixed
-    // end); a non-finite stored value is recorded
-    bool finite = true;
-    auto pull_split = [&](int i, int xs) -> long long {
-        if constexpr (FixedX) {
-            if (xs < 0) return to_fixed(gld[i]);
-            if (xs >= L) return to_fixed(grd[i]);
-        }
-        const float v = float(pull(i, xs));
-        finite &= (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
-        return to_fixed(v);
-    };
-    // x-distance of population i's pull: the rest population streams by k as well
-    auto src_x = [&](auto I) {
-        constexpr int i = decltype(I)::value;
-        constexpr int ex = i == 0 ? 0 : ((i & 1) ? Lat::e((i - 1) / 2, 0) : -Lat::e((i - 1) / 2, 0));
-        return x - (ex + in.kx);
-    };
     bool ok;
     if constexpr (Split) {
-        ok = C::collide_split([&](auto I) { return pull_split(decltype(I)::value, src_x(I)); },
-                              [&](int i, T v) { fout[a.plane[i] + base + x] = v; }, a.wp, a.wlo, a.c,
-                              a.clo, tau_a<T>(in), tau_b<T>(in), mix32(unsigned(base + x) ^ mix32(step)),
-                              in.model, T(in.es_b));
-        ok = ok && finite;
+        // ... in fixed point (the exact double end state beyond a fixed end)
+        float probe = 0.f;  // NaN once a non-finite value has been pulled
+        ok = C::collide_split(
+            [&](int i, const signed char *e, int s, int) -> long long {
+                const int xs = x - (s * e[0] + in.kx);
+                if constexpr (FixedX) {
+                    if (xs < 0) return to_fixed(gld[i]);
+                    if (xs >= L) return to_fixed(grd[i]);
+                }
+                const float v = float(pull(i, xs));
+                probe = __fmaf_rn(v, 0.f, probe);
+                return to_fixed(v);
+            },
+            [&](int i, T v) { fout[a.plane[i] + base + x] = v; }, a.wsh, a.wsl, a.c, a.clo, tau_a<T>(in), tau_b<T>(in),
+            mix32(unsigned(base + x) ^ mix32(step)), in.model, T(in.es_b));
+        ok = ok && probe == 0.f;
     } else {
         T f[Lat::Q];
-        static_for<Lat::Q>([&](auto I) { f[decltype(I)::value] = pull(decltype(I)::value, src_x(I)); });
-        ok = C::collide(f, a.wp, a.wlo, a.c, a.clo, tau_a<T>(in), tau_b<T>(in),
-                        mix32(unsigned(base + x) ^ mix32(step)), in.model, T(in.es_b));
+        static_for<Lat::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            constexpr int ex = i == 0 ? 0 : ((i & 1) ? Lat::e((i - 1) / 2, 0) : -Lat::e((i - 1) / 2, 0));
+            f[i] = pull(i, x - (ex + in.kx));  // the rest population streams by k as well
+        });
+        ok = C::collide(f, a.wp, a.c, tau_a<T>(in), tau_b<T>(in), in.model, T(in.es_b));
         static_for<Lat::Q>([&](auto I) {
             constexpr int i = decltype(I)::value;
             fout[a.plane[i] + base + x] = f[i];
@@ -1093,12 +1140,8 @@ __global__ void __launch_bounds__(128, kStepMinBlocks<Split>) step_line_persiste
 // double, exactly) and wrapped pulls of a periodic line read the state directly.
 template <class Lat>
 struct LineStage {
-    static constexpr int kEmax = [] {
-        int m = 0;
-        for (int p = 0; p < Lat::NP; ++p) m = Lat::e(p, 0) > m ? Lat::e(p, 0) : (-Lat::e(p, 0) > m ? -Lat::e(p, 0) : m);
-        return m;
-    }();
-    static constexpr int kSeg = (32 + 2 * kEmax + 3 + 3) / 4 * 4;  // elements per staged row
+    static constexpr int kEmax = x_reach<Lat>();
+    static constexpr int kSeg = staged_row<Lat>();  // elements per staged row
     static constexpr size_t kRows = size_t(kSeg) * Lat::Q * sizeof(float);
     static constexpr size_t kWarpBytes = 128 + (kRows + 127) / 128 * 128;  // mbarrier, then rows
     SMRT_HD static size_t bytes(int threads) { return size_t(threads / 32) * kWarpBytes; }
@@ -1143,25 +1186,28 @@ SMRT_D bool line_warp_staged(const StepArgs<Lat, float> &a, const float *__restr
     const double *gld = a.ghostsd + (long long)tile.x * 2 * Lat::Q;
     const double *grd = gld + Lat::Q;
     const int tb = int(base + x - in.kx - g_al);  // staged offset of this lane's pull with e_x = 0
-    bool finite = true;
-    auto pullq = [&](auto I) -> long long {
-        constexpr int i = decltype(I)::value;
-        constexpr int ex = i == 0 ? 0 : ((i & 1) ? Lat::e((i - 1) / 2, 0) : -Lat::e((i - 1) / 2, 0));
-        const int xs = x - ex - in.kx;
-        float v;
-        if (xs < 0 || xs >= L) {
-            if constexpr (FixedX) return to_fixed(xs < 0 ? gld[i] : grd[i]);
-            v = load_pop<Coherent>(fin + a.plane[i] + base + wrap(xs, L));
-        } else {
-            v = buf[i * S::kSeg + tb - ex];
+    // does every pull of the warp's cells stay inside the line (warp-uniform)?
+    const int xlast = (xw + 31 < L ? xw + 31 : L - 1);
+    const bool inside = xw - S::kEmax - in.kx >= 0 && xlast + S::kEmax - in.kx < L;
+    float probe = 0.f;  // NaN once a non-finite value has been pulled
+    auto pullq = [&](int i, const signed char *e, int s, int off) -> long long {
+        float v = buf[tb + off];
+        if (!inside) {
+            const int xs = x - s * e[0] - in.kx;
+            if (xs < 0 || xs >= L) {
+                if constexpr (FixedX) return to_fixed(xs < 0 ? gld[i] : grd[i]);
+                v = load_pop<Coherent>(fin + a.plane[i] + base + wrap(xs, L));
+            }
         }
-        finite &= (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
+        probe = __fmaf_rn(v, 0.f, probe);
         return to_fixed(v);
     };
-    const bool ok = C::collide_split(pullq, [&](int i, float v) { fout[a.plane[i] + base + x] = v; }, a.wp, a.wlo,
-                                     a.c, a.clo, tau_a<float>(in), tau_b<float>(in),
-                                     mix32(unsigned(base + x) ^ mix32(step)), in.model, float(in.es_b));
-    if (!(ok && finite)) atomicOr(a.health, 1u);
+    float *dst = fout + base + x;  // library order: plane i starts at i plane[1]
+    const long long stride = a.plane[1];
+    const bool ok = C::collide_split(pullq, [&](int i, float v) { dst[i * stride] = v; }, a.wsh, a.wsl, a.c, a.clo,
+                                     tau_a<float>(in), tau_b<float>(in), mix32(unsigned(base + x) ^ mix32(step)),
+                                     in.model, float(in.es_b));
+    if (!(ok && probe == 0.f)) atomicOr(a.health, 1u);
     return true;
 }
 

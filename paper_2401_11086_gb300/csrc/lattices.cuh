@@ -202,4 +202,79 @@ struct SignOrbits {
 static_assert(SignOrbits<D3Q39>().complete(), "D3Q39 is closed under sign changes");
 static_assert(SignOrbits<D3Q103>().complete(), "D3Q103 is closed under sign changes");
 
+// Largest |e_x| of a set, and the elements per row of a warp's staged x-segment (32 cells, that
+// reach on both sides, rounded out to 16 bytes of floats at either end).
+template <class Lat>
+constexpr int x_reach() {
+    int m = 0;
+    for (int p = 0; p < Lat::NP; ++p) m = Lat::e(p, 0) > m ? Lat::e(p, 0) : (-Lat::e(p, 0) > m ? -Lat::e(p, 0) : m);
+    return m;
+}
+template <class Lat>
+constexpr int staged_row() {
+    return (32 + 2 * x_reach<Lat>() + 3 + 3) / 4 * 4;
+}
+
+// The same orbits as run-time rows for loops over them: grouped by the set of axes on which the
+// orbit's vectors are nonzero (mask: bit d set for axis d), so that within a group every slot's
+// parity class and the slots that do not vanish are the same and stay compile-time, and only the
+// members' population indices, their vectors and the monomials a^gamma are read from the row.
+template <class Lat>
+struct OrbitRows {
+    static constexpr int M = nmom(Lat::NMAX);
+    struct Row {
+        int mono[M];            // a^gamma per slot
+        short ip[4], im[4];     // populations of the member v and of -v
+        short sp[4], sm[4];     // their offsets in a staged segment: population x row - x component
+        signed char e[4][3];    // v
+    };
+    Row row[Lat::NP] = {};
+    int first[9] = {};          // rows [first[mask], first[mask + 1]) belong to mask 1..7
+    static constexpr int mask_of(const SignOrbits<Lat> &s, int o) {
+        int m = 0;
+        for (int t = 0; t < s.k[o]; ++t) m |= 1 << s.ax[o][t];
+        return m;
+    }
+    constexpr OrbitRows() {
+        const SignOrbits<Lat> s;
+        int n = 0;
+        for (int mask = 1; mask < 8; ++mask) {
+            first[mask] = n;
+            for (int o = 0; o < s.n; ++o) {
+                if (mask_of(s, o) != mask) continue;
+                Row &r = row[n++];
+                for (int g = 0; g < M; ++g) r.mono[g] = s.monomial(o, g);
+                for (int b = 0; b < (1 << (s.k[o] - 1)); ++b) {
+                    const int p = s.pair[o][b], fl = s.flip[o][b];
+                    r.ip[b] = short(2 * p + 1 + fl);
+                    r.im[b] = short(2 * p + 2 - fl);
+                    const int vx = fl ? -Lat::e(p, 0) : Lat::e(p, 0);
+                    r.sp[b] = short(r.ip[b] * staged_row<Lat>() - vx);
+                    r.sm[b] = short(r.im[b] * staged_row<Lat>() + vx);
+                    for (int d = 0; d < 3; ++d) r.e[b][d] = (signed char)(fl ? -Lat::e(p, d) : Lat::e(p, d));
+                }
+            }
+        }
+        first[8] = n;
+    }
+    constexpr int count(int mask) const { return first[mask + 1] - first[mask]; }
+};
+constexpr int mask_axes(int mask) { return (mask & 1) + ((mask >> 1) & 1) + (mask >> 2); }
+// does slot g not vanish on the orbits of mask, and its transform entry there: the parities of
+// gamma on the mask's axes after the first
+constexpr bool mask_has(int mask, int g) {
+    for (int d = 0; d < 3; ++d)
+        if (mi_comp(g, d) != 0 && !((mask >> d) & 1)) return false;
+    return true;
+}
+constexpr int mask_class(int mask, int g) {
+    int c = 0, t = 0;
+    for (int d = 0; d < 3; ++d) {
+        if (!((mask >> d) & 1)) continue;
+        if (t > 0 && (mi_comp(g, d) & 1)) c |= 1 << (t - 1);
+        ++t;
+    }
+    return c;
+}
+
 }  // namespace smrt
