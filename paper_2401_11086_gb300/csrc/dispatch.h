@@ -582,7 +582,7 @@ cudaError_t launch_adj_step(const CtxView &v, const void *f, const double *lam_n
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    reduce_partials_kernel<<<1, 32, 0, v.stream>>>(partials, adj_blocks(v), ntau(N), dtau);
+    reduce_partials_kernel<<<1, 32 * ntau(N), 0, v.stream>>>(partials, adj_blocks(v), ntau(N), dtau);
     return cudaGetLastError();
 }
 
@@ -625,7 +625,7 @@ cudaError_t tp_launch_adj_step(const CtxView &v, const void *f, const double *la
         tp_adjoint_step_kernel<L1, N, T, false><<<v.ntiles, 32, 0, v.stream>>>(a, lam_next, lam_t, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    reduce_partials_kernel<<<1, 32, 0, v.stream>>>(partials, (long long)v.ntiles, ntau(N), dtau);
+    reduce_partials_kernel<<<1, 32 * ntau(N), 0, v.stream>>>(partials, (long long)v.ntiles, ntau(N), dtau);
     return cudaGetLastError();
 }
 
