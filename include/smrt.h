@@ -187,7 +187,9 @@ lb_status lb_step(lb_ctx *ctx, void *f_a, void *f_b, int nsteps);
  * 1 selects one block per cell -- its populations in shared memory, the factored sums spread
  * over the block -- which lb_init_lattice picks for problems of at most 48 (LB_F64) or 32 (LB_F32)
  * cells per SM, and
- * which runs one launch per step only);
+ * which runs one launch per step only; on D3Q39 and D3Q103 an LB_F64 context of at most 32 cells
+ * per SM that no schedule has been set on steps with a group of 16 or 32 threads per cell, which
+ * sums in another order than one thread per cell: equal to round-off, not bit for bit);
  * persistent = 1: lb_step runs all its steps in one cooperative launch of blocks_per_sm
  * blocks per SM (0 = as many as fit), tiles spread over the blocks, a grid-wide barrier between
  * steps (its wait is bounded: on timeout the health word gets LB_HEALTH_TIMEOUT and the
@@ -264,8 +266,9 @@ lb_status lb_moments(lb_ctx *ctx, const void *f, double *out, unsigned which_mas
  * beyond a fixed x end are constants (no gradient). The per-block gradient partials live in a
  * scratch array owned by the context; calls on one context must not overlap.
  * Every set has adjoint kernels; on D3Q729 and D3Q4913 the projection of lam_next and the
- * evaluation of the raw moments' adjoint factor over the axes as the forward step does
- * (one thread per cell, 32-cell tiles, the per-tile gradient partials reduced in tile order).
+ * evaluation of the raw moments' adjoint factor over the axes as the forward step does (D3Q39
+ * and D3Q103 lines of at most 32 cells per SM take a group of 16 or 32 threads per cell,
+ * otherwise one thread per cell, 32-cell tiles, the per-tile gradient partials reduced in tile order).
  * Errors: LB_ERR_INVALID (null, lam_next overlapping lam_t, relaxation unset), LB_ERR_UNSUPPORTED
  * (an instance using the ES-BGK model), LB_ERR_CUDA. */
 lb_status lb_step_adjoint(lb_ctx *ctx, const void *f_t, const double *lam_next, double *lam_t,

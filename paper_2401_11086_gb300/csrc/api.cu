@@ -328,13 +328,21 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
     if (e == cudaSuccess) e = cudaMalloc(&c->d_ghostsd, sizeof(double) * c->q * 2 * grid->batch);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_states, sizeof(double) * 10 * grid->batch);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_health, 16);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&c->d_partials, sizeof(double) * kMaxTau * std::max(1LL, line ? c->max_tiles : adj_blocks(v)));
     if (e == cudaSuccess) {
         int dev = 0;
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, dev);
+        v.num_sms = c->num_sms;
     }
+    // a slot per block of the adjoint step: small D3Q39 / D3Q103 lines may take up to
+    // kLaneMaxBlocks blocks of a few cells
+    const bool lane_size = line && !tensor && (long long)ncells <= (long long)kLaneCellsPerSM * c->num_sms;
+    if (e == cudaSuccess)
+        e = cudaMalloc(&c->d_partials,
+                       sizeof(double) * kMaxTau *
+                           std::max(1LL, line ? std::max(c->max_tiles, lane_size ? kLaneMaxBlocks : 0) : adj_blocks(v)));
+    // small double lines step on groups of lanes until a schedule is set
+    v.lanes = line && !tensor && prec == LB_F64 && (long long)ncells <= (long long)kLaneCellsPerSM * c->num_sms;
     // D3Q729 problems of at most 48 (double) or 32 (float) cells per SM take one block per cell
     // (measured crossovers with the tiled kernel)
     if (e == cudaSuccess && c->kind == 2 && (long long)ncells <= (prec == LB_F64 ? 48LL : 32LL) * c->num_sms) {
@@ -606,6 +614,7 @@ extern "C" lb_status lb_set_schedule(lb_ctx *c, const lb_schedule *s) {
     }
     c->sched = *s;
     c->view.tensor_cores = s->tensor_cores;
+    c->view.lanes = 0;
     if (c->sched.persistent && c->ks->occupancy(c->view) < 1) {
         c->sched.persistent = 0;
         return LB_ERR_UNSUPPORTED;

@@ -8,6 +8,7 @@
 #include <cstring>
 
 #include "kernels.cuh"
+#include "lane_kernels.cuh"
 #include "tensor.cuh"
 
 namespace smrt {
@@ -48,6 +49,8 @@ struct CtxView {
     // tensor-product lines: the step kernels' block tiles (instance, first x) of tile_width cells
     const int2 *btiles;
     int nbtiles;
+    int num_sms;
+    int lanes;  // 1: the step of a small double line context runs on groups of lanes (lane_fits)
 };
 
 using StepFn = cudaError_t (*)(const CtxView &, const void *fin, void *fout);
@@ -160,9 +163,61 @@ cudaError_t line_smem_limit() {
     return e;
 }
 
+// The group-of-lanes kernels take grids of at most kLaneCellsPerSM cells per SM; a group is a whole
+// warp up to kLaneWarpCellsPerSM. Measured on 152 SMs, us per step (adjoint step) of one shock, one
+// thread per cell -> lanes; the first column is the same up to 19 k cells:
+//   D3Q39, N = 3    34  -> 14.5 at 400 cells, 16.4 at 1024, 22.5 at 3072, 26.7 at 4096, 37 at 6144
+//   D3Q103, N = 4   92  -> 20.6, 26.7, 39, 49, 91
+//   (adjoint)       237 -> 43, 53, 119, 121, 176
+// and 16 against 32 lanes per cell on D3Q103: 26.0 / 20.8 (53 / 43) at 400 cells, 26.6 / 25.7
+// (53 / 53) at 1024.
+constexpr int kLaneCellsPerSM = 32;
+constexpr int kLaneWarpCellsPerSM = 4;
+constexpr long long kLaneMaxBlocks = 8192;  // of an adjoint step: one slot of partial sums each
+inline int lane_group(const CtxView &v) { return v.ncells <= (long long)kLaneWarpCellsPerSM * v.num_sms ? 32 : 16; }
+inline int lane_blocks_per_tile(const CtxView &v) { return v.tile_width * lane_group(v) / kLaneThreads; }
+// One launch with its dynamic shared memory (more than the default 48 KB: raised once per device
+// and kernel).
+template <auto Kernel>
+cudaError_t lane_smem_limit(size_t bytes) {
+    constexpr int kDevices = 64;
+    static std::atomic<int> state[kDevices];  // 0 not set, 1 set
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
+    if (state[dev].load(std::memory_order_acquire) == 1) return cudaSuccess;
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+    if (e == cudaSuccess) state[dev].store(1, std::memory_order_release);
+    return e;
+}
+
+template <auto Kernel, class Sh, class... A>
+cudaError_t lane_launch(const CtxView &v, const A &...args) {
+    const cudaError_t e = lane_smem_limit<Kernel>(sizeof(Sh));
+    if (e != cudaSuccess) return e;
+    const int bpt = lane_blocks_per_tile(v);
+    Kernel<<<v.ntiles * bpt, kLaneThreads, sizeof(Sh), v.stream>>>(args..., bpt);
+    return cudaGetLastError();
+}
+template <class Lat, int N, bool FixedX, int G>
+cudaError_t lane_step(const CtxView &v, const StepArgs<Lat, double> &a) {
+    return lane_launch<step_lane_kernel<Lat, N, FixedX, G>, LaneShared<Lat, N, false, G>>(v, a);
+}
+template <class Lat, int N, class T, bool FixedX, int G>
+cudaError_t lane_adjoint(const CtxView &v, const StepArgs<Lat, T> &a, const double *in, double *out, double *partials) {
+    return lane_launch<adjoint_lane_kernel<Lat, N, T, FixedX, G>, LaneShared<Lat, N, true, G>>(v, a, in, out, partials);
+}
+
 template <class Lat, int N, class T, class Acc, bool Split>
 cudaError_t launch_step(const CtxView &v, const void *fin, void *fout) {
     const StepArgs<Lat, T> a = make_args<Lat, T>(v, fin, fout);
+    if constexpr (std::is_same<T, double>::value) {
+        if (v.line && v.lanes) {
+            if (lane_group(v) == 32) return v.fixedx ? lane_step<Lat, N, true, 32>(v, a) : lane_step<Lat, N, false, 32>(v, a);
+            return v.fixedx ? lane_step<Lat, N, true, 16>(v, a) : lane_step<Lat, N, false, 16>(v, a);
+        }
+    }
     if constexpr (Split) {
         CUtensorMap map;
         if (v.line && line_encode_map<Lat>(v, fin, &map)) {
@@ -528,12 +583,6 @@ const KernelSet *tp_kernel_set() {
     return &ks;
 }
 
-}  // namespace smrt
-
-#include "adjoint_kernels.cuh"
-
-namespace smrt {
-
 using AdjStepFn = cudaError_t (*)(const CtxView &, const void *f, const double *lam_next, double *lam_t,
                                   double *partials, double *dtau);
 using AdjMomentsFn = cudaError_t (*)(const CtxView &, const void *f, const double *gbar, unsigned mask,
@@ -563,7 +612,13 @@ AdjArgs<Lat, T> make_adj_args(const CtxView &v, const void *f) {
     return A;
 }
 
+// Small line grids (D3Q39, D3Q103) run the adjoint step on groups of lanes.
+inline bool adjoint_on_lanes(const CtxView &v) {
+    return v.line && !v.plane_idx && v.ncells <= (long long)kLaneCellsPerSM * v.num_sms &&
+           (long long)v.ntiles * lane_blocks_per_tile(v) <= kLaneMaxBlocks;
+}
 inline long long adj_blocks(const CtxView &v) {
+    if (adjoint_on_lanes(v)) return (long long)v.ntiles * lane_blocks_per_tile(v);
     return v.line ? (long long)v.ntiles : (long long)((v.nx + kTile - 1) / kTile) * v.ny * v.nz;
 }
 
@@ -574,7 +629,16 @@ cudaError_t launch_adj_step(const CtxView &v, const void *f, const double *lam_n
     A.lam_in = lam_next;
     A.lam_out = lam_t;
     A.partials = partials;
-    if (v.line) {
+    if (adjoint_on_lanes(v)) {
+        cudaError_t el;
+        if (lane_group(v) == 32)
+            el = v.fixedx ? lane_adjoint<Lat, N, T, true, 32>(v, A.s, lam_next, lam_t, partials)
+                          : lane_adjoint<Lat, N, T, false, 32>(v, A.s, lam_next, lam_t, partials);
+        else
+            el = v.fixedx ? lane_adjoint<Lat, N, T, true, 16>(v, A.s, lam_next, lam_t, partials)
+                          : lane_adjoint<Lat, N, T, false, 16>(v, A.s, lam_next, lam_t, partials);
+        if (el != cudaSuccess) return el;
+    } else if (v.line) {
         adjoint_step_kernel<Lat, N, T><<<v.ntiles, v.tile_width, 0, v.stream>>>(A);
     } else {
         const dim3 grid((v.nx + kTile - 1) / kTile, v.ny, v.nz);
