@@ -382,6 +382,7 @@ TPArgs<T> make_tp_args(const CtxView &v, const void *fin, void *fout) {
     a.cd = v.c;
     a.step = v.step;
     a.tma = 0;
+    a.ident = v.plane_identity;
     return a;
 }
 
@@ -460,10 +461,16 @@ cudaError_t tp_launch_step(const CtxView &v, const void *fin, void *fout) {
     TPArgs<T> a = make_tp_args<T>(v, fin, fout);
     if (v.tile_width == 1) {  // one cell per block (D1Q9-P1 sets only: its tables fit in 48 KB)
         if constexpr (L1::Q1 == 9) {
-            if (v.fixedx)
-                tp_step_cell_kernel<L1, N, T, true><<<v.ntiles * 32, 128, 0, v.stream>>>(a);
-            else
-                tp_step_cell_kernel<L1, N, T, false><<<v.ntiles * 32, 128, 0, v.stream>>>(a);
+            if constexpr (std::is_same<T, double>::value) {
+                if (v.fixedx)
+                    tp_step_cell_lanes<L1, N, true><<<v.ntiles * 32, 128, 0, v.stream>>>(a);
+                else
+                    tp_step_cell_lanes<L1, N, false><<<v.ntiles * 32, 128, 0, v.stream>>>(a);
+            } else if (v.fixedx) {
+                tp_step_cell_kernel<L1, N, true><<<v.ntiles * 32, 128, 0, v.stream>>>(a);
+            } else {
+                tp_step_cell_kernel<L1, N, false><<<v.ntiles * 32, 128, 0, v.stream>>>(a);
+            }
             return cudaGetLastError();
         } else {
             return cudaErrorInvalidConfiguration;

@@ -16,6 +16,7 @@ namespace smrt {
 
 static __device__ const LaneMoments<3> kLaneMoments3 = LaneMoments<3>();
 static __device__ const LaneMoments<4> kLaneMoments4 = LaneMoments<4>();
+static __device__ const LaneMoments<5> kLaneMoments5 = LaneMoments<5>();
 static __device__ const LaneOrbits<D3Q39, 3> kLaneOrbits39 = LaneOrbits<D3Q39, 3>();
 static __device__ const LaneOrbits<D3Q103, 3> kLaneOrbits103n3 = LaneOrbits<D3Q103, 3>();
 static __device__ const LaneOrbits<D3Q103, 4> kLaneOrbits103n4 = LaneOrbits<D3Q103, 4>();
@@ -25,6 +26,8 @@ template <>
 SMRT_D const LaneMoments<3> &lane_moments<3>() { return kLaneMoments3; }
 template <>
 SMRT_D const LaneMoments<4> &lane_moments<4>() { return kLaneMoments4; }
+template <>
+SMRT_D const LaneMoments<5> &lane_moments<5>() { return kLaneMoments5; }
 template <class Lat, int N>
 SMRT_D const LaneOrbits<Lat, N> &lane_orbits();
 template <>

@@ -88,16 +88,21 @@ constexpr void fill_pass(Tab &t, int cols, F power) {  // power(row, col) -> j >
 // Sizes of the sparse stages: Hermite conversions (nonzero hfull entries), binomial passes
 // (sum of one component over all slots), traces (three terms per slot of order <= N - 2).
 template <int N>
-constexpr int hermite_nnz() {
+constexpr int hermite_nnz() {  // per component: x^j in He_n for j <= n of its parity
+    const SlotIndex<N> s;
     int n = 0;
-    for (int a = 0; a < nmom(N); ++a)
-        for (int g = 0; g < nmom(N); ++g) n += hfull(a, g) != 0.0;
+    for (int a = 0; a < nmom(N); ++a) {
+        int m = 1;
+        for (int k = 0; k < 3; ++k) m *= s.c[a][k] / 2 + 1;
+        n += m;
+    }
     return n;
 }
 template <int N>
 constexpr int pass_nnz() {
+    const SlotIndex<N> s;
     int n = 0;
-    for (int a = 0; a < nmom(N); ++a) n += mi_comp(a, 0);
+    for (int a = 0; a < nmom(N); ++a) n += s.c[a][0];
     return n;
 }
 
@@ -116,7 +121,7 @@ struct alignas(16) LaneMoments {
     SparseRows<M2, 3 * M2> delT;         // its transpose
     SparseRows<kC, kC * (N / 2 + 1)> cj; // C[n][j] = sum_m B(n,m) D(n-2m, j-m) s_(n,m)
     SparseRows<ntau(N), kC * (N / 2 + 1)> cjT;
-    unsigned char ord[M] = {};
+    unsigned char ord[M] = {}, comp[M][4] = {};  // order, components of a slot
     // ES-BGK target of order 4: ordered pairs of order-2 slots adding up to the slot
     unsigned char es_n[M] = {}, es_q1[M][8] = {}, es_q2[M][8] = {};
     // pairs of slots p = q + j e_k, by j: pairs [gbeg[j], gbeg[j + 1]) of gp[k], gq[k]
@@ -125,13 +130,19 @@ struct alignas(16) LaneMoments {
     SMRT_HD static constexpr int c_slot(int n, int j) { return (n - 2) * (N / 2 + 1) + j; }
     constexpr LaneMoments() {
         const SlotIndex<N> s;
-        for (int p = 0; p < M; ++p) ord[p] = (unsigned char)s.ord[p];
+        for (int p = 0; p < M; ++p) {
+            ord[p] = (unsigned char)s.ord[p];
+            for (int k = 0; k < 3; ++k) comp[p][k] = (unsigned char)s.c[p][k];
+        }
+        double h1[N + 1][N + 1] = {}, fa[N + 1] = {};
+        for (int n = 0; n <= N; ++n) {
+            fa[n] = fact_small(n);
+            for (int j = 0; j <= n; ++j) h1[n][j] = he_coef_l(n, j);
+        }
         auto he = [&](int a, int g) {  // hfull
-            double h = 1.0;
-            for (int k = 0; k < 3; ++k) h *= he_coef_l(s.c[a][k], s.c[g][k]);
-            return h;
+            return h1[s.c[a][0]][s.c[g][0]] * h1[s.c[a][1]][s.c[g][1]] * h1[s.c[a][2]][s.c[g][2]];
         };
-        auto af = [&](int a) { return fact_small(s.c[a][0]) * fact_small(s.c[a][1]) * fact_small(s.c[a][2]); };
+        auto af = [&](int a) { return fa[s.c[a][0]] * fa[s.c[a][1]] * fa[s.c[a][2]]; };
         fill_rows(hd, M, [&](int a, int g) { return he(a, g) / af(a); });
         fill_rows(hf, M, [&](int a, int g) { return he(a, g); });
         fill_rows(hdT, M, [&](int g, int a) { return he(a, g) / af(a); });

@@ -22,7 +22,7 @@
 
 
 #include "kernels.cuh"
-#include "moment_tables.cuh"
+#include "lane_kernels.cuh"
 
 namespace smrt {
 
@@ -66,6 +66,7 @@ struct TPArgs {
     double cd;                         // lattice scale c
     unsigned step;
     int tma;                           // 1: the kernel's tensor maps describe fin and fout
+    int ident;                         // 1: library population i is caller plane i
 };
 
 // Tensor maps of the two states for the block-staged kernels: a 2D view [plane][stride] of a
@@ -383,151 +384,6 @@ struct TPCell {
         binomial_divided<N, T>(v, G);
         v[0] = rhom1;  // deviation from the coefficients of w_i
         to_rebuild(v, c, R);
-        return ok;
-    }
-
-    // The steps of collide_moments (a2, a4-a6) with one cell's coefficients spread over the 32
-    // lanes of a warp: lane l owns slots l and l + 32, each step reads the whole vector from
-    // shared memory and writes its own slots (the per-slot constants come from MomentTables).
-    // Executing the single-thread version on every lane would spend a full warp's FP64 issue
-    // on each scalar operation. R (shared, M values): raw moments in, rebuild coefficients out;
-    // w (shared, M values) and gs (shared, 3 (N + 1) values): scratch. Every lane calls it.
-    SMRT_D static bool collide_moments_lanes(const MomentSmem<N, double> &tb, T *R, T *w, T *gs, T c, const T *tauA,
-                                             const T *tauB, int model, T es_b) {
-        const int lane = threadIdx.x & 31;
-        const int pa = lane, pb = lane + 32;
-        const bool two = pb < M;
-        // the lane's slots: components and orders in registers
-        const int ca[3] = {tb.c[pa][0], tb.c[pa][1], tb.c[pa][2]};
-        const int cb[3] = {two ? tb.c[pb][0] : 0, two ? tb.c[pb][1] : 0, two ? tb.c[pb][2] : 0};
-        const int oa = tb.c[pa][3], ob = two ? tb.c[pb][3] : 0;
-        auto ipow_t = [](T x, int e) {
-            T r = T(1);
-            for (int i = 0; i < e; ++i) r *= x;
-            return r;
-        };
-        auto axis_pass = [&](const T *src, T *dst, int k) {  // dst = T_k src (one binomial axis)
-            auto one = [&](int p, const int (&cc)[3]) {
-                const int ak = cc[k];
-                T acc = src[p];
-                for (int b = 0; b < ak; ++b) {
-                    const int q = k == 0 ? mi_pos(b, cc[1], cc[2]) : (k == 1 ? mi_pos(cc[0], b, cc[2]) : mi_pos(cc[0], cc[1], b));
-                    acc = fma(gs[k * (N + 1) + ak - b], src[q], acc);
-                }
-                dst[p] = acc;
-            };
-            one(pa, ca);
-            if (two) one(pb, cb);
-            __syncwarp();
-        };
-        // Rc = c^|gamma| R
-        w[pa] = R[pa] * ipow_t(c, oa);
-        if (two) w[pb] = R[pb] * ipow_t(c, ob);
-        __syncwarp();
-        // a2 (every lane): rho - 1 = Rc_0, rho u = Rc_1, E - 3 = tr Rc_2
-        const T rhom1 = w[0];
-        const T rho = T(1) + rhom1;
-        const T ir = rcp(rho);
-        const T u0 = w[mi_pos(1, 0, 0)] * ir, u1 = w[mi_pos(0, 1, 0)] * ir, u2 = w[mi_pos(0, 0, 1)] * ir;
-        const T uu = u0 * u0 + u1 * u1 + u2 * u2;
-        const T thm1 = (w[mi_pos(2, 0, 0)] + w[mi_pos(0, 2, 0)] + w[mi_pos(0, 0, 2)] - T(3) * rhom1 - rho * uu) * ir *
-                       T(1.0 / 3.0);
-        const T theta = T(1) + thm1;
-        const bool ok = (rho > T(0)) && (theta > T(0));
-        // ta = hdiv Rc (into R), full a_0 = rho
-        auto hd_row = [&](int p) {
-            T acc = T(0);
-            for (int i = 0; i < tb.hd_n[p]; ++i) acc = fma(tb.hd_val[p][i], w[tb.hd_col[p][i]], acc);
-            R[p] = p == 0 ? rho : acc;
-        };
-        hd_row(pa);
-        if (two) hd_row(pb);
-        // a4: T(-u, 2 - theta) then theta^(-|beta|/2)
-        if (lane < 3) {
-            T G[N + 1];
-            maxwell_divided<N, T>(G, lane == 0 ? -u0 : (lane == 1 ? -u1 : -u2), -thm1);
-            for (int j = 0; j <= N; ++j) gs[lane * (N + 1) + j] = G[j];
-        }
-        __syncwarp();
-        axis_pass(R, w, 0);
-        axis_pass(w, R, 1);
-        axis_pass(R, w, 2);
-        const T is = rsq(theta);
-        w[pa] *= ipow_t(is, oa);
-        if (two) w[pb] *= ipow_t(is, ob);
-        __syncwarp();
-        // a5: w -> R
-        if (model == 1) {
-            const T tau = fma(tauB[0], rho, tauA[0]) * ir;
-            const T om = rcp(tau);
-            const T bp = T(1) - (T(1) - es_b) * tau * rcp(fma(T(-0.5), es_b, tau));
-            const T sr = T(1) - om, s2 = fma(om, bp, sr), k4 = om * bp * bp * T(0.5) * ir;
-            auto es_slot = [&](int p, int n) {
-                T v = w[p];
-                if (n == 2) {
-                    v *= s2;
-                } else if (n == 4) {
-                    T t4 = T(0);
-                    for (int i = 0; i < tb.es_n[p]; ++i) t4 = fma(w[tb.es_q1[p][i]], w[tb.es_q2[p][i]], t4);
-                    v = fma(k4, t4, sr * v);
-                } else if (n >= 3) {
-                    v *= sr;
-                }
-                R[p] = v;
-            };
-            es_slot(pa, oa);
-            if (two) es_slot(pb, ob);
-        } else {
-            auto smrt_slot = [&](int p, int n) {
-                if (n < 2) {
-                    R[p] = w[p];
-                    return;
-                }
-                const int k0 = tau_slot(n, 0);  // s_m for m = 0, 1, 2 (n <= 5)
-                const T s0 = T(1) - rcp_tau<T>(tauA[k0], tauB[k0], rho);
-                const T s1 = T(1) - rcp_tau<T>(tauA[k0 + 1], tauB[k0 + 1], rho);
-                const T s2 = n >= 4 ? T(1) - rcp_tau<T>(tauA[k0 + 2], tauB[k0 + 2], rho) : T(0);
-                const int len = (n + 1) * (n + 2) / 2, o = ord_off(n), lp = p - o;
-                T acc = s0 * w[p];  // C_0 = s_0 B(n,0) D(n,0) = s_0
-                for (int j = 1; j <= n / 2; ++j) {
-                    T Cj = s0 * T(tb.bd[n][j][0]);
-                    Cj = fma(s1, T(tb.bd[n][j][1]), Cj);
-                    if (j >= 2) Cj = fma(s2, T(tb.bd[n][j][2]), Cj);
-                    const T *row = tb.rel + RelaxTables<N>::off(n, j) + lp * len;
-                    T dot = T(0);
-                    for (int q = 0; q < len; ++q) dot = fma(row[q], w[o + q], dot);
-                    acc = fma(Cj, dot, acc);
-                }
-                R[p] = acc;
-            };
-            smrt_slot(pa, oa);
-            if (two) smrt_slot(pb, ob);
-        }
-        // a6: theta^(|beta|/2), order 0 = rho, order 1 = 0, then T(u, theta)
-        const T sq = theta * is;
-        auto back_scale = [&](int p, int n) { R[p] = n == 0 ? rho : (n == 1 ? T(0) : R[p] * ipow_t(sq, n)); };
-        back_scale(pa, oa);
-        if (two) back_scale(pb, ob);
-        if (lane < 3) {
-            T G[N + 1];
-            maxwell_divided<N, T>(G, lane == 0 ? u0 : (lane == 1 ? u1 : u2), thm1);
-            for (int j = 0; j <= N; ++j) gs[lane * (N + 1) + j] = G[j];
-        }
-        __syncwarp();
-        axis_pass(R, w, 0);
-        axis_pass(w, R, 1);
-        axis_pass(R, w, 2);
-        if (lane == 0) w[0] = rhom1;  // deviation from the coefficients of w_i
-        __syncwarp();
-        // P_gamma = c^|gamma| sum_alpha hfull(alpha, gamma) ta_alpha (into R)
-        auto hf_row = [&](int p, int n) {
-            T acc = T(0);
-            for (int i = 0; i < tb.hf_n[p]; ++i) acc = fma(tb.hf_val[p][i], w[tb.hf_col[p][i]], acc);
-            R[p] = acc * ipow_t(c, n);
-        };
-        hf_row(pa, oa);
-        if (two) hf_row(pb, ob);
-        __syncwarp();
         return ok;
     }
 
@@ -1104,35 +960,27 @@ __global__ void __launch_bounds__(128) tp_step_line_persistent_block(TPArgs<T> a
 // ------------------------------------------------------------------ one cell per block
 // For problems too small to fill the GPU with one thread per cell (the paper's own runs are
 // single shocks of 100 cells), each block takes one cell: its d^3 pulled populations go to
-// shared memory, the x-rows and the raw moments are summed by the block's threads, the
-// moment-space steps run in warp 0 with the coefficients spread over its lanes, and the
-// rebuild is spread over the x-rows again. Block b takes cell x0 + b % 32 of the 32-cell tile b / 32.
-template <class L1, int N, class T>
+// shared memory, the x-rows and the raw moments are summed by the block's threads, and the
+// rebuild is spread over them again. Block b takes cell x0 + b % 32 of the 32-cell tile b / 32.
+//
+// Float: the moment-space steps run on one thread, whose compile-time constants beat tables.
+template <class L1, int N>
 struct TPCellShared {
     static constexpr int Q1 = L1::Q1, P2 = Q1 * Q1, Q = P2 * Q1, M = nmom(N);
-    T f[Q];             // pulled populations, library order
-    T g[P2][N + 1];     // x-row sums g_j of row (b, c) = b + d c
-    T ep[Q1][N + 1];    // e_a^j
-    T R[M];             // raw moments, then the rebuild coefficients
-    T h[Q1][N + 1][N + 1];  // per z-plane c: sum over y of the x-row sums (then of the rebuild)
-    T w[M];             // moment-space scratch
-    T gs[3 * (N + 1)];  // per-axis Maxwellian coefficients of the frame transforms
+    float f[Q];             // pulled populations, library order
+    float g[P2][N + 1];     // x-row sums g_j of row (b, c) = b + d c
+    float ep[Q1][N + 1];    // e_a^j
+    float R[M];             // raw moments, then the rebuild coefficients
+    float h[Q1][N + 1][N + 1];  // per z-plane c: sum over y of the x-row sums (then of the rebuild)
 };
 
-template <class L1, int N, class T, bool FixedX>
-__global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<T> a) {
-    using C = TPCell<L1, N, T>;
-    using SH = TPCellShared<L1, N, T>;
+template <class L1, int N, bool FixedX>
+__global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<float> a) {
+    using C = TPCell<L1, N, float>;
+    using SH = TPCellShared<L1, N>;
     constexpr int Q1 = SH::Q1, P2 = SH::P2, Q = SH::Q, M = SH::M;
-    __shared__ TPTables<L1, T> s;
+    __shared__ TPTables<L1, float> s;
     __shared__ SH sh;
-    // double: the moment-space steps spread over warp 0's lanes need their tables in shared
-    // memory (a redundant full-warp FP64 instruction costs a full warp of the FP64 pipe); float
-    // keeps the one-thread form, whose compile-time constants beat the tables' latency
-    constexpr bool kLanes = std::is_same<T, double>::value;
-    struct NoTables {};
-    __shared__ typename std::conditional<kLanes, MomentSmem<N, double>, NoTables>::type ms;
-    if constexpr (kLanes) load_moment_smem<N>(ms);
     tp_load_tables<L1>(a, s);  // ends with __syncthreads
     const int tid = threadIdx.x;
     const int2 tile = a.tiles[blockIdx.x >> 5];
@@ -1140,18 +988,18 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<T> a) {
     const int x = tile.y + int(blockIdx.x & 31u), L = in.nx, kx = in.kx;
     if (x >= L) return;  // the whole block: no barrier follows for it
     const long long base = in.cell_off;
-    const T *gl = a.ghosts + (long long)tile.x * 2 * Q;
-    const T *gr = gl + Q;
+    const float *gl = a.ghosts + (long long)tile.x * 2 * Q;
+    const float *gr = gl + Q;
     for (int q = tid; q < Q1 * (N + 1); q += blockDim.x) {
         const int av = q / (N + 1), j = q % (N + 1);
-        T p = T(1);
+        float p = 1.f;
         for (int r = 0; r < j; ++r) p *= s.e[av];
         sh.ep[av][j] = p;
     }
     // a1: pull every population of the cell
     for (int i = tid; i < Q; i += blockDim.x) {
         const int t = x - e1<L1>(i % Q1) - kx;
-        T v;
+        float v;
         if (FixedX && t < 0)
             v = gl[i];
         else if (FixedX && t >= L)
@@ -1163,9 +1011,9 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<T> a) {
     __syncthreads();
     // a3, x first: one x-row per thread
     for (int row = tid; row < P2; row += blockDim.x) {
-        const T *fr = sh.f + row * Q1;
-        T g[N + 1];
-        C::xrow([&](auto A) -> T { return fr[decltype(A)::value]; }, g);
+        const float *fr = sh.f + row * Q1;
+        float g[N + 1];
+        C::xrow([&](auto A) -> float { return fr[decltype(A)::value]; }, g);
         static_for<N + 1>([&](auto J) { sh.g[row][decltype(J)::value] = g[decltype(J)::value]; });
     }
     __syncthreads();
@@ -1174,7 +1022,7 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<T> a) {
     for (int q = tid; q < Q1 * JK; q += blockDim.x) {
         const int c = q / JK, j = (q % JK) / (N + 1), k = q % (N + 1);
         if (j + k > N) continue;
-        T acc = T(0);
+        float acc = 0.f;
         for (int b = 0; b < Q1; ++b) acc = fma(sh.g[b + Q1 * c][j], sh.ep[b][k], acc);
         sh.h[c][j][k] = acc;
     }
@@ -1182,26 +1030,20 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<T> a) {
     // ... then z: R_(j,k,l) = sum_c h_c(j,k) e_c^l, one moment per thread
     for (int m = tid; m < M; m += blockDim.x) {
         const int j = mi_comp(m, 0), k = mi_comp(m, 1), l = mi_comp(m, 2);
-        T acc = T(0);
+        float acc = 0.f;
         for (int c = 0; c < Q1; ++c) acc = fma(sh.h[c][j][k], sh.ep[c][l], acc);
         sh.R[m] = acc;
     }
     __syncthreads();
     // a2, a4-a6 in warp 0
     if (tid < 32) {
-        if constexpr (kLanes) {
-            const bool ok = C::collide_moments_lanes(ms, sh.R, sh.w, sh.gs, T(a.cd), tau_a<T>(in),
-                                                     tau_b<T>(in), in.model, T(in.es_b));
-            if (tid == 0 && !ok) atomicOr(a.health, 1u);
-        } else {
-            T R[M];
-            static_for<M>([&](auto G) { R[decltype(G)::value] = sh.R[decltype(G)::value]; });
-            const bool ok = C::collide_moments(R, T(a.cd), tau_a<T>(in), tau_b<T>(in), in.model, T(in.es_b));
-            __syncwarp();
-            if (tid == 0) {
-                if (!ok) atomicOr(a.health, 1u);
-                static_for<M>([&](auto G) { sh.R[decltype(G)::value] = R[decltype(G)::value]; });
-            }
+        float R[M];
+        static_for<M>([&](auto G) { R[decltype(G)::value] = sh.R[decltype(G)::value]; });
+        const bool ok = C::collide_moments(R, float(a.cd), tau_a<float>(in), tau_b<float>(in), in.model, float(in.es_b));
+        __syncwarp();
+        if (tid == 0) {
+            if (!ok) atomicOr(a.health, 1u);
+            static_for<M>([&](auto G) { sh.R[decltype(G)::value] = R[decltype(G)::value]; });
         }
     }
     __syncthreads();
@@ -1209,28 +1051,207 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<T> a) {
     for (int q = tid; q < Q1 * JK; q += blockDim.x) {
         const int c = q / JK, j = (q % JK) / (N + 1), k = q % (N + 1);
         if (j + k > N) continue;
-        T acc = T(0);
+        float acc = 0.f;
         for (int l = 0; l + j + k <= N; ++l) acc = fma(sh.R[mi_pos(j, k, l)], sh.ep[c][l], acc);
         sh.h[c][j][k] = acc;
     }
     __syncthreads();
     // ... then one x-row per thread, Pb_j = sum_k Pc_c(j,k) e_b^k, stored as it is formed
-    T *dst = a.fout + base + x;
-    auto put = [&](int i, T v) { dst[(long long)s.plane[i] * a.stride] = v; };
+    float *dst = a.fout + base + x;
+    auto put = [&](int i, float v) { dst[(long long)s.plane[i] * a.stride] = v; };
     for (int row = tid; row < P2; row += blockDim.x) {
         const int b = row % Q1, c = row / Q1;
-        T Pb[N + 1];
+        float Pb[N + 1];
         static_for<N + 1>([&](auto J) {
             constexpr int j = decltype(J)::value;
-            T acc = T(0);
+            float acc = 0.f;
             static_for<N + 1 - j>([&](auto K) {
                 constexpr int k = decltype(K)::value;
                 acc = fma(sh.h[c][j][k], sh.ep[b][k], acc);
             });
             Pb[j] = acc;
         });
-        C::template emit_x<T>(Pb, s.w[b] * s.w[c], s.w, row * Q1, put);
+        C::template emit_x<float>(Pb, s.w[b] * s.w[c], s.w, row * Q1, put);
     }
+}
+
+// Double: every stage is spread over the block's threads, the moment-space steps as the sparse
+// stages of lane_cell.cuh on two warps (a full-warp FP64 instruction holds a quarter of the SM's
+// FP64 pipe for 64 cycles whether or not its lanes do useful work, so what counts is the number of
+// instructions in a row, not the number of lanes they use). One 100-cell shock, N = 5: 46 us per
+// step with the moment space on one warp in dense order blocks, 22.8 us here (371 us on the
+// block-staged kernel); 4800 cells 204 us (373).
+struct TPCellGroup {
+    static constexpr int G = 64;
+    int lane;
+    SMRT_D void sync() const { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+};
+template <class L1, int N, bool Adjoint>
+struct TPLaneShared {
+    static constexpr int Q1 = L1::Q1, P2 = Q1 * Q1, Q = P2 * Q1, M = nmom(N);
+    static constexpr int kJK = (N + 1) * (N + 2) / 2;  // (j, k) with j + k <= N
+    using C = LaneCell<N>;
+    LaneMoments<N> m;
+    double f[(Q + 1) / 2 * 2];      // populations, library order (the adjoint: then lam's)
+    double g[P2][N + 1];            // x-row sums g_j of row b + d c; x-row coefficients of the rebuild
+    double pw[Q1][N + 1];           // e_a^j
+    double w[Q1 + 1];
+    double h[Q1][kJK];              // per z-plane c: sums over y; plane coefficients of the rebuild
+    double cp[N + 1 + (N & 1 ? 0 : 1)];
+    double V[Adjoint ? int(C::kAdjoint) : int(C::kForward)];
+    // (j, k) of index r, j ascending then k, three bits each
+    SMRT_HD static constexpr unsigned long long packed(bool second) {
+        unsigned long long v = 0;
+        int r = 0;
+        for (int j = 0; j <= N; ++j)
+            for (int k = 0; k + j <= N; ++k, ++r) v |= (unsigned long long)(second ? k : j) << (3 * r);
+        return v;
+    }
+    SMRT_D static int j_of(int r) {
+        constexpr unsigned long long v = packed(false);
+        return int((v >> (3 * r)) & 7ull);
+    }
+    SMRT_D static int k_of(int r) {
+        constexpr unsigned long long v = packed(true);
+        return int((v >> (3 * r)) & 7ull);
+    }
+    SMRT_D static int jk(int j, int k) { return j * (N + 1) - j * (j - 1) / 2 + k; }
+    // The sums of the populations in f: c-scaled raw moments into R (shared). All threads of the
+    // block; ends with a block barrier.
+    SMRT_D void project(double *R) {
+        using T = TPCell<L1, N, double>;
+        for (int row = threadIdx.x; row < P2; row += blockDim.x) {
+            const double *fr = f + row * Q1;
+            double gr[N + 1];
+            T::xrow([&](auto A) -> double { return fr[decltype(A)::value]; }, gr);
+            static_for<N + 1>([&](auto J) { g[row][decltype(J)::value] = gr[decltype(J)::value]; });
+        }
+        __syncthreads();
+        // y, +-e_b folded: h_c(j,k) = sum_b g_(b,c)j e_b^k
+        for (int q = threadIdx.x; q < Q1 * kJK; q += blockDim.x) {
+            const int c = q / kJK, r = q % kJK, j = j_of(r), k = k_of(r);
+            double acc = k == 0 ? g[Q1 * c][j] : 0.0;
+#pragma unroll
+            for (int p = 0; p < L1::NP1; ++p) {
+                const double gp = g[Q1 * c + 2 * p + 1][j], gm = g[Q1 * c + 2 * p + 2][j];
+                acc = fma(pw[2 * p + 1][k], (k & 1) ? gp - gm : gp + gm, acc);
+            }
+            h[c][r] = acc;
+        }
+        __syncthreads();
+        // z, +-e_c folded: one moment per thread
+        for (int q = threadIdx.x; q < M; q += blockDim.x) {
+            const int r = jk(m.comp[q][0], m.comp[q][1]), l = m.comp[q][2];
+            double acc = l == 0 ? h[0][r] : 0.0;
+#pragma unroll
+            for (int p = 0; p < L1::NP1; ++p) {
+                const double hp = h[2 * p + 1][r], hm = h[2 * p + 2][r];
+                acc = fma(pw[2 * p + 1][l], (l & 1) ? hp - hm : hp + hm, acc);
+            }
+            R[q] = acc * cp[m.ord[q]];
+        }
+        __syncthreads();
+    }
+    // Populations from the (c-scaled) coefficients P (shared): put(i, value without the weights).
+    // All threads; P ready on entry.
+    template <class Put>
+    SMRT_D void rebuild(const double *P, Put &&put) {
+        for (int q = threadIdx.x; q < Q1 * kJK; q += blockDim.x) {
+            const int c = q / kJK, r = q % kJK, j = j_of(r), k = k_of(r);
+            double acc = P[mi_pos(j, k, 0)];
+            for (int l = 1; l + j + k <= N; ++l) acc = fma(P[mi_pos(j, k, l)], pw[c][l], acc);
+            h[c][r] = acc;
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < P2 * (N + 1); q += blockDim.x) {
+            const int row = q % P2, j = q / P2, b = row % Q1, c = row / Q1, r = jk(j, 0);
+            double acc = h[c][r];
+            for (int k = 1; k + j <= N; ++k) acc = fma(h[c][r + k], pw[b][k], acc);
+            g[row][j] = acc;
+        }
+        __syncthreads();
+        // one +-e_a pair (or the rest velocity) of a row per thread
+        for (int q = threadIdx.x; q < P2 * (L1::NP1 + 1); q += blockDim.x) {
+            const int row = q % P2, p = q / P2;
+            const double *G = g[row];
+            if (p == L1::NP1) {
+                put(row * Q1, G[0]);
+            } else {
+                const double *e = pw[2 * p + 1];
+                double ev = fma(e[2], G[2], G[0]), od = e[1] * G[1];
+                od = fma(e[3], G[3], od);
+                ev = fma(e[4], G[4], ev);
+                if constexpr (N >= 5) od = fma(e[5], G[5], od);
+                put(row * Q1 + 2 * p + 1, ev + od);
+                put(row * Q1 + 2 * p + 2, ev - od);
+            }
+        }
+    }
+    // tables of the block (no barrier)
+    template <class T>
+    SMRT_D void load(const TPArgs<T> &a) {
+        lane_copy(m, lane_moments<N>());
+        if (threadIdx.x < Q1) {
+            const double ea = e1<L1>(threadIdx.x);
+            double p = 1.0;
+            for (int k = 0; k <= N; ++k, p *= ea) pw[threadIdx.x][k] = p;
+            w[threadIdx.x] = a.w1[threadIdx.x];
+        } else if (threadIdx.x == 32) {
+            double p = 1.0;
+            for (int k = 0; k <= N; ++k, p *= a.cd) cp[k] = p;
+        }
+    }
+    SMRT_D double weight(int i) const { return w[i % Q1] * w[i / Q1 % Q1] * w[i / P2]; }
+};
+
+template <class L1, int N, bool FixedX>
+__global__ void __launch_bounds__(128) tp_step_cell_lanes(TPArgs<double> a) {
+    using SH = TPLaneShared<L1, N, false>;
+    constexpr int Q1 = SH::Q1, Q = SH::Q;
+    __shared__ __align__(16) unsigned char raw[sizeof(SH)];
+    SH &s = *reinterpret_cast<SH *>(raw);
+    const int tid = threadIdx.x;
+    const int2 tile = a.tiles[blockIdx.x >> 5];
+    const InstanceInfo &in = a.inst[tile.x];
+    const int x = tile.y + int(blockIdx.x & 31u), L = in.nx, kx = in.kx;
+    if (x >= L) return;  // the whole block
+    const long long base = in.cell_off;
+    const double *gl = a.ghosts + (long long)tile.x * 2 * Q;
+    auto plane = [&](int i) -> long long { return (a.ident ? i : __ldg(a.plane_idx + i)) * a.stride + base; };
+    // a1: the pulls and the tables, all in flight together
+    constexpr int kPer = (Q + 127) / 128;
+    double v[kPer];
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+        const int i = tid + 128 * r;
+        v[r] = 0.0;
+        if (i < Q) {
+            const int t = x - e1<L1>(i % Q1) - kx;
+            if (FixedX && t < 0)
+                v[r] = gl[i];
+            else if (FixedX && t >= L)
+                v[r] = gl[Q + i];
+            else
+                v[r] = a.fin[plane(i) + (FixedX ? t : wrap(t, L))];
+        }
+    }
+    s.load(a);
+#pragma unroll
+    for (int r = 0; r < kPer; ++r)
+        if (tid + 128 * r < Q) s.f[tid + 128 * r] = v[r];
+    __syncthreads();
+    s.project(s.V + LaneCell<N>::oRc);
+    double *P = s.V + LaneCell<N>::oTa;
+    if (tid < TPCellGroup::G) {
+        const TPCellGroup g{tid};
+        LaneCell<N> cell;
+        const bool ok = cell.collide(s.m, g, s.V, in.tauA, in.tauB, in.model, in.es_b,
+                                     [&](int k, double c) { P[k] = c * s.cp[s.m.ord[k]]; });
+        if (tid == 0 && !ok) atomicOr(a.health, 1u);
+    }
+    __syncthreads();
+    double *dst = a.fout + x;
+    s.rebuild(P, [&](int i, double c) { dst[plane(i)] = c * s.weight(i); });
 }
 
 // lb_moments of the pulled (pre-collision) populations.
