@@ -490,6 +490,15 @@ cudaError_t tp_launch_step(const CtxView &v, const void *fin, void *fout) {
 template <class L1, int N, class T>
 cudaError_t tp_launch_moments(const CtxView &v, const void *f, double *out, unsigned mask) {
     const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
+    // small double problems: one block per cell, as the step
+    if constexpr (L1::Q1 == 9 && std::is_same<T, double>::value)
+        if (v.ncells <= 48ll * v.num_sms) {
+            if (v.fixedx)
+                tp_moments_cell_lanes<L1, N, true><<<v.ntiles * 32, 128, 0, v.stream>>>(a, out, v.ncells, mask);
+            else
+                tp_moments_cell_lanes<L1, N, false><<<v.ntiles * 32, 128, 0, v.stream>>>(a, out, v.ncells, mask);
+            return cudaGetLastError();
+        }
     tp_moments_kernel<L1, N, T><<<v.ntiles, 32, 0, v.stream>>>(a, out, v.ncells, mask, v.fixedx);
     return cudaGetLastError();
 }

@@ -139,13 +139,11 @@ struct LaneCell {
         return rho > 0.0 && th > 0.0;
     }
 
-    // F2 - F6: V's raw moments to td, td', y, q1, q2 (F6's last pass is left to the callers).
-    // model 1: ES-BGK with parameter es_b. False when rho or theta is not positive.
+    // F2 - F4: V's raw moments to the local-frame coefficients td; G of both transforms. False when
+    // rho or theta is not positive.
     template <class Group>
-    SMRT_HD bool forward(const Tab &t, const Group &g, double *V, const double *tauA, const double *tauB, int model,
-                         double es_b) {
+    SMRT_HD bool local(const Tab &t, const Group &g, double *V) {
         const bool ok = conserved(V);
-        // F3; the G of both transforms; the relaxation factors
         rows(t.hd, g, V + oRc, [&](int a, double v) { V[oTa + a] = a == 0 ? rho : v; });
         for (int r = g.lane; r < 6; r += Group::G) {
             const double uk = r < 3 ? -u_of(r) : u_of(r - 3), t1 = r < 3 ? -thm1 : thm1;
@@ -160,17 +158,27 @@ struct LaneCell {
                 b = n;
             }
         }
-        for (int k = g.lane; k < KT; k += Group::G) {
+        g.sync();
+        pass(t.pass[0], g, g_of(V, 0, 0), V + oTa, V + oP1);
+        pass(t.pass[1], g, g_of(V, 0, 1), V + oP1, V + oP2);
+        pass(t.pass[2], g, g_of(V, 0, 2), V + oP2, [&](int p, double v) { V[oTd + p] = v * V[oPw + t.ord[p]]; });
+        return ok;
+    }
+
+    // F2 - F6: V's raw moments to td, td', y, q1, q2 (F6's last pass is left to the callers).
+    // model 1: ES-BGK with parameter es_b. False when rho or theta is not positive.
+    template <class Group>
+    SMRT_HD bool forward(const Tab &t, const Group &g, double *V, const double *tauA, const double *tauB, int model,
+                         double es_b) {
+        const bool ok = local(t, g, V);
+        for (int k = g.lane; k < KT; k += Group::G) {  // the relaxation factors
             const double R = 1.0 / fma(tauB[k], rho, tauA[k]);
             V[oS + KT + k] = R;
             V[oS + k] = 1.0 - rho * R;
         }
         g.sync();
         rows(t.cj, g, V + oS, [&](int c, double v) { V[oC + c] = v; });
-        // F4
-        pass(t.pass[0], g, g_of(V, 0, 0), V + oTa, V + oP1);
-        pass(t.pass[1], g, g_of(V, 0, 1), V + oP1, V + oP2);
-        pass(t.pass[2], g, g_of(V, 0, 2), V + oP2, [&](int p, double v) { V[oTd + p] = v * V[oPw + t.ord[p]]; });
+        g.sync();
         // F5
         if (model == 1) {
             const double tau = fma(tauB[0], rho, tauA[0]) * ir, om = 1.0 / tau;

@@ -1201,6 +1201,30 @@ struct TPLaneShared {
             for (int k = 0; k <= N; ++k, p *= a.cd) cp[k] = p;
         }
     }
+    // the cell's pulled populations and the tables, all in flight together (no barrier)
+    template <bool FixedX, class T, class Plane>
+    SMRT_D void pull(const TPArgs<T> &a, const T *gl, int x, int L, int kx, Plane &&plane) {
+        constexpr int kPer = (Q + 127) / 128;
+        T v[kPer];
+#pragma unroll
+        for (int r = 0; r < kPer; ++r) {
+            const int i = threadIdx.x + 128 * r;
+            v[r] = T(0);
+            if (i < Q) {
+                const int t = x - e1<L1>(i % Q1) - kx;
+                if (FixedX && t < 0)
+                    v[r] = gl[i];
+                else if (FixedX && t >= L)
+                    v[r] = gl[Q + i];
+                else
+                    v[r] = a.fin[plane(i) + (FixedX ? t : wrap(t, L))];
+            }
+        }
+        load(a);
+#pragma unroll
+        for (int r = 0; r < kPer; ++r)
+            if (threadIdx.x + 128 * r < Q) f[threadIdx.x + 128 * r] = double(v[r]);
+    }
     SMRT_D double weight(int i) const { return w[i % Q1] * w[i / Q1 % Q1] * w[i / P2]; }
 };
 
@@ -1218,27 +1242,7 @@ __global__ void __launch_bounds__(128) tp_step_cell_lanes(TPArgs<double> a) {
     const long long base = in.cell_off;
     const double *gl = a.ghosts + (long long)tile.x * 2 * Q;
     auto plane = [&](int i) -> long long { return (a.ident ? i : __ldg(a.plane_idx + i)) * a.stride + base; };
-    // a1: the pulls and the tables, all in flight together
-    constexpr int kPer = (Q + 127) / 128;
-    double v[kPer];
-#pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-        const int i = tid + 128 * r;
-        v[r] = 0.0;
-        if (i < Q) {
-            const int t = x - e1<L1>(i % Q1) - kx;
-            if (FixedX && t < 0)
-                v[r] = gl[i];
-            else if (FixedX && t >= L)
-                v[r] = gl[Q + i];
-            else
-                v[r] = a.fin[plane(i) + (FixedX ? t : wrap(t, L))];
-        }
-    }
-    s.load(a);
-#pragma unroll
-    for (int r = 0; r < kPer; ++r)
-        if (tid + 128 * r < Q) s.f[tid + 128 * r] = v[r];
+    s.template pull<FixedX>(a, gl, x, L, kx, plane);
     __syncthreads();
     s.project(s.V + LaneCell<N>::oRc);
     double *P = s.V + LaneCell<N>::oTa;
@@ -1252,6 +1256,35 @@ __global__ void __launch_bounds__(128) tp_step_cell_lanes(TPArgs<double> a) {
     __syncthreads();
     double *dst = a.fout + x;
     s.rebuild(P, [&](int i, double c) { dst[plane(i)] = c * s.weight(i); });
+}
+
+// lb_moments on the same blocks (double; the small problems above). The paper's 100-cell shock:
+// 208 -> 20 us, one thread per cell being 4 warps on the whole GPU.
+template <class L1, int N, bool FixedX>
+__global__ void __launch_bounds__(128) tp_moments_cell_lanes(TPArgs<double> a, double *out, long long ncells, unsigned mask) {
+    using SH = TPLaneShared<L1, N, false>;
+    using C = LaneCell<N>;
+    __shared__ __align__(16) unsigned char raw[sizeof(SH)];
+    SH &s = *reinterpret_cast<SH *>(raw);
+    const int2 tile = a.tiles[blockIdx.x >> 5];
+    const InstanceInfo &in = a.inst[tile.x];
+    const int x = tile.y + int(blockIdx.x & 31u), L = in.nx, kx = in.kx;
+    if (x >= L) return;  // the whole block
+    const long long base = in.cell_off;
+    s.template pull<FixedX>(a, a.ghosts + (long long)tile.x * 2 * SH::Q, x, L, kx, [&](int i) -> long long {
+        return (a.ident ? i : __ldg(a.plane_idx + i)) * a.stride + base;
+    });
+    __syncthreads();
+    s.project(s.V + C::oRc);
+    if (threadIdx.x >= TPCellGroup::G) return;
+    const TPCellGroup g{int(threadIdx.x)};
+    C cell;
+    cell.local(s.m, g, s.V);
+    if (threadIdx.x != 0) return;
+    const double up[3] = {cell.u[0] + a.cd * in.kx, cell.u[1], cell.u[2]};
+    double v[C::M];
+    for (int p = 0; p < C::M; ++p) v[p] = s.V[C::oTd + p];
+    store_moments<N, double>(out, ncells, base + x, mask, cell.rho, up, cell.th, v);
 }
 
 // lb_moments of the pulled (pre-collision) populations.
