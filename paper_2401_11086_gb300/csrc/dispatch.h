@@ -366,7 +366,7 @@ const KernelSet *kernel_set() {
 }
 
 // ------------------------------------------------------------------ tensor-product sets
-template <class T>
+template <class L1, class T>
 TPArgs<T> make_tp_args(const CtxView &v, const void *fin, void *fout) {
     TPArgs<T> a;
     a.fin = static_cast<const T *>(fin);
@@ -458,7 +458,7 @@ cudaError_t tp_launch_block_w(const CtxView &v, const TPArgs<T> &a, const void *
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_step(const CtxView &v, const void *fin, void *fout) {
-    TPArgs<T> a = make_tp_args<T>(v, fin, fout);
+    TPArgs<T> a = make_tp_args<L1, T>(v, fin, fout);
     if (v.tile_width == 1) {  // one cell per block (D1Q9-P1 sets only: its tables fit in 48 KB)
         if constexpr (L1::Q1 == 9) {
             if constexpr (std::is_same<T, double>::value) {
@@ -489,7 +489,7 @@ cudaError_t tp_launch_step(const CtxView &v, const void *fin, void *fout) {
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_moments(const CtxView &v, const void *f, double *out, unsigned mask) {
-    const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
+    const TPArgs<T> a = make_tp_args<L1, T>(v, f, nullptr);
     // small double problems: one block per cell, as the step
     if constexpr (L1::Q1 == 9 && std::is_same<T, double>::value)
         if (v.ncells <= 48ll * v.num_sms) {
@@ -505,14 +505,14 @@ cudaError_t tp_launch_moments(const CtxView &v, const void *f, double *out, unsi
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_fill(const CtxView &v, void *f, const double *rho, const double *u, const double *theta) {
-    const TPArgs<T> a = make_tp_args<T>(v, nullptr, f);
+    const TPArgs<T> a = make_tp_args<L1, T>(v, nullptr, f);
     tp_fill_kernel<L1, N, T><<<v.ntiles, 32, 0, v.stream>>>(a, rho, u, theta, v.ncells);
     return cudaGetLastError();
 }
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_ghost(const CtxView &v, const double *states, int ninst, void *ghosts, double *ghostsd) {
-    const TPArgs<T> a = make_tp_args<T>(v, nullptr, nullptr);
+    const TPArgs<T> a = make_tp_args<L1, T>(v, nullptr, nullptr);
     const int n = 2 * ninst;
     tp_ghost_kernel<L1, N, T><<<(n + 63) / 64, 64, 0, v.stream>>>(a, states, ninst, static_cast<T *>(ghosts), ghostsd);
     return cudaGetLastError();
@@ -566,7 +566,7 @@ cudaError_t tp_persist_block_w(const CtxView &v, const TPArgs<T> &a, void *fa, v
 // occ non-null: report the resident blocks per SM instead of launching
 template <class L1, int N, class T>
 cudaError_t tp_persist_dispatch(const CtxView &v, void *fa, void *fb, int nsteps, int grid, int *occ) {
-    const TPArgs<T> a = make_tp_args<T>(v, fa, fb);
+    const TPArgs<T> a = make_tp_args<L1, T>(v, fa, fb);
     if constexpr (std::is_same<T, float>::value)
         if (v.fixedx && v.tensor_cores)
             return v.plane_identity ? tp_persist_block_w<L1, N, T, true, true, true>(v, a, fa, fb, nsteps, grid, occ)
@@ -698,7 +698,7 @@ namespace smrt {
 template <class L1, int N, class T>
 cudaError_t tp_launch_adj_step(const CtxView &v, const void *f, const double *lam_next, double *lam_t,
                                double *partials, double *dtau) {
-    const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
+    const TPArgs<T> a = make_tp_args<L1, T>(v, f, nullptr);
     if (v.fixedx)
         tp_adjoint_step_kernel<L1, N, T, true><<<v.ntiles, 32, 0, v.stream>>>(a, lam_next, lam_t, partials);
     else
@@ -711,7 +711,7 @@ cudaError_t tp_launch_adj_step(const CtxView &v, const void *f, const double *la
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_adj_moments(const CtxView &v, const void *f, const double *gbar, unsigned mask, double *lam) {
-    const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
+    const TPArgs<T> a = make_tp_args<L1, T>(v, f, nullptr);
     if (v.fixedx)
         tp_adjoint_moments_kernel<L1, N, T, true><<<v.ntiles, 32, 0, v.stream>>>(a, gbar, mask, lam, v.ncells);
     else
