@@ -91,18 +91,22 @@ struct AdjMoments {
     SMRT_HD static void maxwell(double u, double t, double (&G)[Nm + 1]) {
         G[0] = 1.0;
         G[1] = u;
-        for (int j = 1; j < Nm; ++j) G[j + 1] = (u * G[j] + t * G[j - 1]) / (j + 1);
+        static_for<Nm - 1>([&](auto J) {
+            constexpr int j = decltype(J)::value + 1;
+            G[j + 1] = (u * G[j] + t * G[j - 1]) * (1.0 / (j + 1));
+        });
     }
     // transpose of maxwell: consumes Gb, accumulates ub and tb
     SMRT_HD static void maxwell_T(double u, double t, const double (&G)[Nm + 1], double (&Gb)[Nm + 1],
                                   double &ub, double &tb) {
-        for (int j = Nm - 1; j >= 1; --j) {
-            const double g = Gb[j + 1] / (j + 1);
+        static_for<Nm - 1>([&](auto J) {
+            constexpr int j = Nm - 1 - decltype(J)::value;
+            const double g = Gb[j + 1] * (1.0 / (j + 1));
             ub += g * G[j];
             Gb[j] += g * u;
             tb += g * G[j - 1];
-            Gb[j - 1] += g * t;
-        }
+            if constexpr (j > 1) Gb[j - 1] += g * t;  // Gb[0] is not read
+        });
         ub += Gb[1];
     }
 
@@ -122,6 +126,7 @@ struct AdjMoments {
             }
         });
     }
+    // Xb_q += sum_p (tr)_(p,q) Zb_p over the orders r of X (r = 2..most; Zb of order r - 2)
     template <int r>
     SMRT_HD static void tr_T(const double (&Zb)[M], double (&Xb)[M]) {
         static_for<M>([&](auto A) {
@@ -134,6 +139,7 @@ struct AdjMoments {
             }
         });
     }
+    // W_p += (delta Y)_p, p of order r
     template <int r>
     SMRT_HD static void delta(const double (&Y)[M], double (&W)[M]) {
         static_for<M>([&](auto A) {
@@ -144,84 +150,74 @@ struct AdjMoments {
                     constexpr int k = decltype(K)::value;
                     if constexpr (mi_comp(p, k) >= 2) acc += Y[mi_minus2(p, k)];
                 });
-                W[p] = acc / double(r * (r - 1));
+                W[p] += acc * (1.0 / (r * (r - 1)));
             }
         });
     }
+    // Yb of order r - 2 = the transpose of delta<r> on Wb
     template <int r>
     SMRT_HD static void delta_T(const double (&Wb)[M], double (&Yb)[M]) {
         static_for<M>([&](auto A) {
             constexpr int p = decltype(A)::value;
-            if constexpr (mi_order(p) == r) {
-                static_for<3>([&](auto K) {
-                    constexpr int k = decltype(K)::value;
-                    if constexpr (mi_comp(p, k) >= 2) Yb[mi_minus2(p, k)] += Wb[p] / double(r * (r - 1));
-                });
+            if constexpr (mi_order(p) == r - 2) {
+                const double acc = Wb[mi_plus2(p, 0)] + Wb[mi_plus2(p, 1)] + Wb[mi_plus2(p, 2)];
+                Yb[p] = acc * (1.0 / (r * (r - 1)));
             }
         });
     }
 
-    // L_j td = delta^j tr^j td restricted to order n (full-slot arrays, other orders untouched)
-    template <int n, int j>
-    SMRT_HD static void lift(const double (&td)[M], double (&out)[M]) {
-        double cur[M];
-        static_for<M>([&](auto A) { cur[decltype(A)::value] = td[decltype(A)::value]; });
-        static_for<j>([&](auto I) {
-            constexpr int r = n - 2 * decltype(I)::value;
-            double nxt[M];
-            tr<r>(cur, nxt);
-            static_for<M>([&](auto A) {
-                constexpr int p = decltype(A)::value;
-                if constexpr (mi_order(p) == r - 2) cur[p] = nxt[p];
-            });
-        });
-        static_for<j>([&](auto I) {
-            constexpr int r = n - 2 * j + 2 * (decltype(I)::value + 1);
-            double nxt[M];
-            delta<r>(cur, nxt);
-            static_for<M>([&](auto A) {
-                constexpr int p = decltype(A)::value;
-                if constexpr (mi_order(p) == r) cur[p] = nxt[p];
-            });
-        });
+    // F5 on order n: sum_j C_j delta^j tr^j td (J = n / 2 <= 2 traces), as C_0 td + delta z,
+    // z = C_1 t1 + C_2 delta t2 with t1 = tr td, t2 = tr t1, which the transpose reads again. All in
+    // the slots of their own orders of full-slot arrays.
+    template <int n>
+    SMRT_HD static void relax(const double (&td)[M], const double (&C)[3], double (&t1)[M], double (&t2)[M],
+                              double (&tdp)[M]) {
+        static_assert(Nm <= 5 && n <= Nm, "at most two traces");
+        double z[M];
+        tr<n>(td, t1);
+        if constexpr (n >= 4) tr<n - 2>(t1, t2);
         static_for<M>([&](auto A) {
             constexpr int p = decltype(A)::value;
-            if constexpr (mi_order(p) == n) out[p] = cur[p];
+            if constexpr (mi_order(p) == n - 2) z[p] = n >= 4 ? 0.0 : C[1] * t1[p];
         });
+        if constexpr (n >= 4) {
+            delta<n - 2>(t2, z);
+            static_for<M>([&](auto A) {
+                constexpr int p = decltype(A)::value;
+                if constexpr (mi_order(p) == n - 2) z[p] = C[2] * z[p] + C[1] * t1[p];
+            });
+        }
+        static_for<M>([&](auto A) {
+            constexpr int p = decltype(A)::value;
+            if constexpr (mi_order(p) == n) tdp[p] = C[0] * td[p];
+        });
+        delta<n>(z, tdp);
     }
-    // L_j^T wb (order n) accumulated into tdb (order n)
-    template <int n, int j>
-    SMRT_HD static void lift_T(const double (&wb)[M], double (&tdb)[M]) {
-        double cur[M];
-        static_for<M>([&](auto A) { cur[decltype(A)::value] = 0.0; });
+    // its transpose: tdb (order n) from tdpb, and the adjoints of the C_j:
+    // w1 = delta^T tdpb, w2 = delta^T w1, tdb = C_0 tdpb + tr^T (C_1 w1 + C_2 tr^T w2),
+    // Cb = (tdpb.td, w1.t1, w2.t2)
+    template <int n>
+    SMRT_HD static void relax_T(const double (&tdpb)[M], const double (&td)[M], const double (&t1)[M],
+                                const double (&t2)[M], const double (&C)[3], double (&tdb)[M], double (&Cb)[3]) {
+        double w1[M], w2[M], x[M];
+        Cb[0] = Cb[1] = Cb[2] = 0.0;
+        delta_T<n>(tdpb, w1);
+        if constexpr (n >= 4) delta_T<n - 2>(w1, w2);
         static_for<M>([&](auto A) {
             constexpr int p = decltype(A)::value;
-            if constexpr (mi_order(p) == n) cur[p] = wb[p];
+            if constexpr (mi_order(p) == n) {
+                Cb[0] += tdpb[p] * td[p];
+                tdb[p] = C[0] * tdpb[p];
+            } else if constexpr (mi_order(p) == n - 2) {
+                Cb[1] += w1[p] * t1[p];
+                x[p] = C[1] * w1[p];
+            } else if constexpr (n >= 4 && mi_order(p) == n - 4) {
+                Cb[2] += w2[p] * t2[p];
+                w2[p] *= C[2];
+            }
         });
-        static_for<j>([&](auto I) {  // delta^T from order n down to n - 2j
-            constexpr int r = n - 2 * decltype(I)::value;
-            double nxt[M];
-            static_for<M>([&](auto A) { nxt[decltype(A)::value] = 0.0; });
-            delta_T<r>(cur, nxt);
-            static_for<M>([&](auto A) {
-                constexpr int p = decltype(A)::value;
-                if constexpr (mi_order(p) == r - 2) cur[p] = nxt[p];
-            });
-        });
-        static_for<j>([&](auto I) {  // tr^T from order n - 2j up to n
-            constexpr int r = n - 2 * j + 2 * (decltype(I)::value + 1);
-            double nxt[M];
-            static_for<M>([&](auto A) { nxt[decltype(A)::value] = 0.0; });
-            tr_T<r>(cur, nxt);
-            static_for<M>([&](auto A) {
-                constexpr int p = decltype(A)::value;
-                if constexpr (mi_order(p) == r) cur[p] = nxt[p];
-            });
-        });
-        static_for<M>([&](auto A) {
-            constexpr int p = decltype(A)::value;
-            if constexpr (mi_order(p) == n) tdb[p] += cur[p];
-        });
+        if constexpr (n >= 4) tr_T<n - 2>(w2, x);
+        tr_T<n>(x, tdb);
     }
 };
 
@@ -343,29 +339,29 @@ struct AdjMath : AdjMoments<Nm> {
 // Conserved moments from the raw moments (F2) and the transpose of F2 (onto Rcb).
 template <int M>
 struct Conserved {
-    double rho, rhom1, u[3], thm1, th;
+    double rho, rhom1, ir, u[3], uu, thm1, th;
     SMRT_HD void from_raw(const double (&Rc)[M]) {
         rhom1 = Rc[0];
         rho = 1.0 + rhom1;
-        u[0] = Rc[mi_pos(1, 0, 0)] / rho;
-        u[1] = Rc[mi_pos(0, 1, 0)] / rho;
-        u[2] = Rc[mi_pos(0, 0, 1)] / rho;
-        const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+        ir = 1.0 / rho;
+        u[0] = Rc[mi_pos(1, 0, 0)] * ir;
+        u[1] = Rc[mi_pos(0, 1, 0)] * ir;
+        u[2] = Rc[mi_pos(0, 0, 1)] * ir;
+        uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         const double em3 = Rc[mi_pos(2, 0, 0)] + Rc[mi_pos(0, 2, 0)] + Rc[mi_pos(0, 0, 2)];
-        thm1 = (em3 - 3.0 * rhom1 - rho * uu) / (3.0 * rho);
+        thm1 = (em3 - 3.0 * rhom1 - rho * uu) * (ir * (1.0 / 3.0));
         th = 1.0 + thm1;
     }
     // rhob collects every adjoint of rho (and of rho - 1); ub, tb those of u and theta - 1
     SMRT_HD void transpose(double rhob, const double (&ub)[3], double tb, double (&Rcb)[M]) const {
-        const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        Rcb[0] += rhob - (ub[0] * u[0] + ub[1] * u[1] + ub[2] * u[2]) / rho +
-                  tb * ((uu - 3.0) / (3.0 * rho) - thm1 / rho);
-        Rcb[mi_pos(1, 0, 0)] += ub[0] / rho - tb * 2.0 * u[0] / (3.0 * rho);
-        Rcb[mi_pos(0, 1, 0)] += ub[1] / rho - tb * 2.0 * u[1] / (3.0 * rho);
-        Rcb[mi_pos(0, 0, 1)] += ub[2] / rho - tb * 2.0 * u[2] / (3.0 * rho);
-        Rcb[mi_pos(2, 0, 0)] += tb / (3.0 * rho);
-        Rcb[mi_pos(0, 2, 0)] += tb / (3.0 * rho);
-        Rcb[mi_pos(0, 0, 2)] += tb / (3.0 * rho);
+        const double t3 = tb * ir * (1.0 / 3.0);
+        Rcb[0] += rhob - (ub[0] * u[0] + ub[1] * u[1] + ub[2] * u[2]) * ir + t3 * (uu - 3.0) - tb * thm1 * ir;
+        Rcb[mi_pos(1, 0, 0)] += ub[0] * ir - 2.0 * t3 * u[0];
+        Rcb[mi_pos(0, 1, 0)] += ub[1] * ir - 2.0 * t3 * u[1];
+        Rcb[mi_pos(0, 0, 1)] += ub[2] * ir - 2.0 * t3 * u[2];
+        Rcb[mi_pos(2, 0, 0)] += t3;
+        Rcb[mi_pos(0, 2, 0)] += t3;
+        Rcb[mi_pos(0, 0, 2)] += t3;
     }
 };
 
@@ -415,25 +411,21 @@ SMRT_HD void moment_vjp(const double (&Rc)[nmom(N)], const double (&Lc)[nmom(N)]
         R[k] = 1.0 / (tauA[k] + tauB[k] * rho);
         s[k] = 1.0 - rho * R[k];
     }
-    // relaxation: td'_n = sum_j C_j L_j td_n; keep L_j td_n for the C_j adjoints
-    double tdp[M];
-    static_for<M>([&](auto A) { tdp[decltype(A)::value] = 0.0; });
-    double Lj[N + 1][N / 2 + 1][M];
+    // relaxation: td'_n = sum_j C_j delta^j tr^j td_n, C_j = sum_{m<=j} s_m B(n,m) D(n-2m, j-m)
+    double tdp[M], t1s[M], t2s[M], C[N + 1][3];
     static_for<N - 1>([&](auto Nn) {
         constexpr int n = decltype(Nn)::value + 2;
-        static_for<n / 2 + 1>([&](auto Jj) {
+        static_for<3>([&](auto Jj) {
             constexpr int j = decltype(Jj)::value;
-            AM::template lift<n, j>(td, Lj[n][j]);
             double Cj = 0.0;
-            static_for<j + 1>([&](auto Mm) {
+            static_for<(j <= n / 2 ? j + 1 : 0)>([&](auto Mm) {
                 constexpr int m = decltype(Mm)::value;
                 Cj += coefB(n, m) * coefD(n - 2 * m, j - m) * s[tau_slot(n, m)];
             });
-            static_for<M>([&](auto A) {
-                constexpr int p = decltype(A)::value;
-                if constexpr (mi_order(p) == n) tdp[p] += Cj * Lj[n][j][p];
-            });
+            C[n][j] = Cj;
         });
+        // t1 of order n - 2, t2 of order n - 4: no two orders n share a slot
+        AM::template relax<n>(td, C[n], t1s, t2s, tdp);
     });
     double y[M];
     static_for<M>([&](auto A) {
@@ -468,46 +460,32 @@ SMRT_HD void moment_vjp(const double (&Rc)[nmom(N)], const double (&Lc)[nmom(N)]
     AM::template pass_T<1>(q2b, Gp[1], q1, q1b, Gb[1]);
     AM::template pass_T<0>(q1b, Gp[0], y, yb, Gb[0]);
     for (int k = 0; k < 3; ++k) AM::maxwell_T(cs.u[k], t1, Gp[k], Gb[k], ub[k], tb);
-    // F6'
+    // F6'; ts: the theta adjoint's sums per order, d theta^(n/2) / d theta = n/2 theta^(n/2) / theta
     rhob += yb[0];
-    double tdpb[M];
+    double tdpb[M], ts[N + 1];
+    for (int n = 0; n <= N; ++n) ts[n] = 0.0;
     static_for<M>([&](auto A) {
         constexpr int p = decltype(A)::value;
         constexpr int o = mi_order(p);
         if constexpr (o >= 2) {
             tdpb[p] = yb[p] * sqp[o];
-            tb += yb[p] * tdp[p] * (0.5 * o) * sqp[o] / th;
+            ts[o] += tdpb[p] * tdp[p];
         } else {
             tdpb[p] = 0.0;
         }
     });
     // F5'
     double tdb[M], sb[KT];
-    static_for<M>([&](auto A) { tdb[decltype(A)::value] = 0.0; });
     for (int k = 0; k < KT; ++k) sb[k] = 0.0;
     static_for<N - 1>([&](auto Nn) {
         constexpr int n = decltype(Nn)::value + 2;
+        double Cb[3];
+        AM::template relax_T<n>(tdpb, td, t1s, t2s, C[n], tdb, Cb);
         static_for<n / 2 + 1>([&](auto Jj) {
             constexpr int j = decltype(Jj)::value;
-            double Cj = 0.0, Cjb = 0.0;
             static_for<j + 1>([&](auto Mm) {
                 constexpr int m = decltype(Mm)::value;
-                Cj += coefB(n, m) * coefD(n - 2 * m, j - m) * s[tau_slot(n, m)];
-            });
-            double scaled[M];
-            static_for<M>([&](auto A) {
-                constexpr int p = decltype(A)::value;
-                if constexpr (mi_order(p) == n) {
-                    Cjb += tdpb[p] * Lj[n][j][p];
-                    scaled[p] = Cj * tdpb[p];
-                } else {
-                    scaled[p] = 0.0;
-                }
-            });
-            AM::template lift_T<n, j>(scaled, tdb);
-            static_for<j + 1>([&](auto Mm) {
-                constexpr int m = decltype(Mm)::value;
-                sb[tau_slot(n, m)] += coefB(n, m) * coefD(n - 2 * m, j - m) * Cjb;
+                sb[tau_slot(n, m)] += coefB(n, m) * coefD(n - 2 * m, j - m) * Cb[j];
             });
         });
     });
@@ -523,11 +501,16 @@ SMRT_HD void moment_vjp(const double (&Rc)[nmom(N)], const double (&Lc)[nmom(N)]
         p2b[p] = p1b[p] = tab[p] = 0.0;
         if constexpr (o >= 2) {
             p3b[p] = tdb[p] * isp[o];
-            tb -= tdb[p] * p3[p] * (0.5 * o) * isp[o] / th;
+            ts[o] -= tdb[p] * td[p];
         } else {
             p3b[p] = 0.0;
         }
     });
+    {
+        double tsum = 0.0;
+        for (int n = 2; n <= N; ++n) tsum += 0.5 * n * ts[n];
+        tb += tsum / th;
+    }
     double Gmb[3][N + 1];
     for (int k = 0; k < 3; ++k)
         for (int j = 0; j <= N; ++j) Gmb[k][j] = 0.0;

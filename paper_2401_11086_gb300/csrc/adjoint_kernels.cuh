@@ -155,7 +155,7 @@ static __global__ void __launch_bounds__(32 * kMaxTau) reduce_partials_kernel(co
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= kt) return;
     double acc = 0.0;
-#pragma unroll 4
+#pragma unroll 8
     for (long long b = lane; b < nblocks; b += 32) acc += partials[b * kt + k];
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
     if (lane == 0) dtau[k] += acc;
