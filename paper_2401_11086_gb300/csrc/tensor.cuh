@@ -128,6 +128,36 @@ SMRT_D void tp_load_tables(const TPArgs<T> &a, TPTables<L1, U, Planes> &s) {
     __syncthreads();
 }
 
+// Two floats in one 64-bit register pair: one packed instruction (add / multiply / fused
+// multiply-add, each lane rounded as the scalar one) works on both.
+struct F2 {
+    unsigned long long v;
+    F2() = default;
+    SMRT_D F2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    SMRT_D F2(float a) : F2(a, a) {}
+    SMRT_D F2(double a) : F2(float(a), float(a)) {}
+    SMRT_D F2(int a) : F2(float(a), float(a)) {}
+    SMRT_D float lo() const { return __uint_as_float(static_cast<unsigned>(v)); }
+    SMRT_D float hi() const { return __uint_as_float(static_cast<unsigned>(v >> 32)); }
+    // friends: found for F2 arguments only (fma of floats and doubles stays the global one)
+    SMRT_D friend F2 operator+(F2 a, F2 b) {
+        F2 r;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+        return r;
+    }
+    SMRT_D friend F2 operator*(F2 a, F2 b) {
+        F2 r;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+        return r;
+    }
+    SMRT_D friend F2 fma(F2 a, F2 b, F2 c) {
+        F2 r;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+        return r;
+    }
+    SMRT_D friend F2 operator-(F2 a, F2 b) { return fma(F2(-1.f), b, a); }
+};
+
 template <class L1, int N, class T>
 struct TPCell {
     static constexpr int Q1 = L1::Q1;
@@ -442,7 +472,7 @@ struct TPCell {
     // f'_(a,b,c) = w (ev +- E od), od the odd part over E; w: w_a w_b w_c by the class of a.
     template <class U, class W, class Put>
     SMRT_D static void emit_x(const U (&Pb)[N + 1], const W &w, int i0, Put &put) {
-        put(i0, w[0] * Pb[0]);
+        put(i0, U(w[0]) * Pb[0]);
         static_for<NP1>([&](auto Q) {
             constexpr int q = decltype(Q)::value, E = L1::E(q);
             U ev = Pb[0], od = Pb[1];
@@ -554,13 +584,12 @@ struct TPBlockStage {
     static constexpr int kEmax = L1::E(L1::NP1 - 1);    // largest |e| of the 1D rule
     static constexpr int kSeg = kW + ((2 * kEmax + kAlign - 1) + kAlign - 1) / kAlign * kAlign;
     static_assert(kSeg <= 256, "a tensor-map box spans at most 256 elements");
-    // a stage buffer holds two groups of d rows (the +e_b and -e_b x-rows), each group
-    // starting 128-byte aligned so that one tensor-map box fills it
-    static constexpr int kGrp = int((L1::Q1 * kSeg * sizeof(T) + 127) / 128 * 128 / sizeof(T));
-    // then the end-state populations of the stage's planes, [left, right][2 d], for the pulls
-    // from beyond a line's fixed ends
-    static constexpr int kGhost = int((4 * L1::Q1 * sizeof(T) + 127) / 128 * 128 / sizeof(T));
-    static constexpr int kStage = 2 * kGrp + kGhost;    // elements per stage buffer
+    // a stage buffer holds two groups of d rows (the +e_b and -e_b x-rows), each group starting
+    // 128-byte aligned so that one tensor-map box fills it, and after its rows the end-state
+    // populations of its planes, [left, right][d], for the pulls from beyond a line's fixed ends
+    static constexpr int kEnds = L1::Q1 * kSeg;
+    static constexpr int kGrp = int(((kEnds + 2 * L1::Q1) * sizeof(T) + 127) / 128 * 128 / sizeof(T));
+    static constexpr int kStage = 2 * kGrp;             // elements per stage buffer
     static constexpr int kPerZ = L1::NP1 + 1;           // stages per z-plane
     static constexpr int kTotal = L1::Q1 * kPerZ;       // stages per step
     static_assert(kTotal % kStages == 0, "each tile starts the buffers' cycle at buffer 0");
@@ -741,11 +770,11 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
         if constexpr (Coherent) fence_async_global();
         fence_async_shared();
         if (needL || needR) {  // the stage's end-state populations ride along with its fill
-            T *gs = sbuf + 2 * S::kGrp;
             const int i0 = cz * P2 + k0;
             for (int k = lane; k < nplanes; k += 32) {
-                if (needL) cp_async_elem(gs + k, gl + i0 + k);
-                if (needR) cp_async_elem(gs + 2 * Q1 + k, gr + i0 + k);
+                T *gs = sbuf + S::kEnds + (k < Q1 ? k : S::kGrp + k - Q1);
+                if (needL) cp_async_elem(gs, gl + i0 + k);
+                if (needR) cp_async_elem(gs + Q1, gr + i0 + k);
             }
             cp_async_mbar_arrive(b);
             __syncwarp();  // before lane 0's arrival below can complete the phase
@@ -775,15 +804,22 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
     // the lane's pull by x-velocity a of a staged row sits at row + a SEG + tb - e_a; each
     // (plane, slot) is read by this lane only, so the lane may overwrite its own slots
     const int tb = int(base + x - kx - g_al);
-    // pulls from beyond the line's ends: their slots get what the pull must see (the end
-    // state's population, or the wrapped population of a periodic line) once the fill lands
-    unsigned beyond = 0u;
+    // pulls from beyond the line's ends, by x-velocity (bit a). Fixed ends: such a pull reads the
+    // end state staged after the group's rows; a warp none of whose cells has one reads the rows
+    // directly. (Rewriting the lanes' slots in the staged rows instead, one diverged branch per
+    // velocity and stage, took an edge warp 62 k cycles per tile where the sums take 15 k.) The wrapped
+    // pulls of a periodic line, and the operands of the tensor cores, are rewritten in the rows.
+    unsigned beyL = 0u, beyR = 0u;
     if (active)
         static_for<Q1>([&](auto A) {
             constexpr int av = decltype(A)::value;
             const int t = x - e1<L1>(av) - kx;
-            if (t < 0 || t >= L) beyond |= 1u << av;
+            if (t < 0) beyL |= 1u << av;
+            if (t >= L) beyR |= 1u << av;
         });
+    const unsigned beyond = beyL | beyR;
+    constexpr bool kRewrite = TC || !FixedX;
+    const bool edge = !kRewrite && __any_sync(0xffffffffu, beyond != 0u);
     if (warp == 0)
         for (int st = 0; st < NS; ++st)
             if (!issue(st)) return fail();
@@ -806,7 +842,7 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
         pending &= ~(1u << sb);
         const int cz = st / S::kPerZ, p = st % S::kPerZ;
         T *bs = buf + size_t(sb) * S::kStage;
-        if (active && beyond) {
+        if (kRewrite && active && beyond) {
             const int nrows = p ? 2 : 1;
             const int k0 = p ? (2 * p - 1) * Q1 : 0;
             static_for<Q1>([&](auto A) {
@@ -816,7 +852,7 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
                     for (int r = 0; r < nrows; ++r) {
                         T v;
                         if constexpr (FixedX)  // the end state's population, staged with the fill
-                            v = bs[2 * S::kGrp + (t < 0 ? 0 : 2 * Q1) + r * Q1 + av];
+                            v = bs[r * S::kGrp + S::kEnds + (t < 0 ? 0 : Q1) + av];
                         else
                             v = load_pop<Coherent>(fin + plane(cz * P2 + k0 + r * Q1 + av) * a.stride + base +
                                                    wrap(t, L));
@@ -840,26 +876,42 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
             if (active && p == NP1) C::zfold_pw(h, s.pw[cz], R);
             fence_async_shared();  // scratch written and read: before the buffer's next fill
         } else if (active) {
-            const T *r0 = bs + tb;
-            auto rowp = [&](auto A) -> T {
-                constexpr int av = decltype(A)::value;
-                return r0[av * SEG - e1<L1>(av)];
+            // at(ic<a>): the stage offset of the lane's pull by x-velocity a in the group of +e_b
+            auto sums = [&](auto &&at) {
+                if (p == 0) {
+                    T g[N + 1];
+                    C::xrow([&](auto A) -> T { return bs[at(A)]; }, g);
+                    C::yrest(g, h);
+                } else {
+                    T gp[N + 1], gm[N + 1];
+                    if constexpr (std::is_same<T, float>::value) {  // both rows in packed pairs
+                        F2 g2[N + 1];
+                        TPCell<L1, N, F2>::xrow(
+                            [&](auto A) -> F2 {
+                                const int o = at(A);
+                                return F2(bs[o], bs[o + S::kGrp]);
+                            },
+                            g2);
+                        static_for<N + 1>([&](auto J) {
+                            gp[decltype(J)::value] = g2[decltype(J)::value].lo();
+                            gm[decltype(J)::value] = g2[decltype(J)::value].hi();
+                        });
+                    } else {
+                        C::xrow([&](auto A) -> T { return bs[at(A)]; }, gp);
+                        C::xrow([&](auto A) -> T { return bs[at(A) + S::kGrp]; }, gm);
+                    }
+                    C::ypair_pw(gp, gm, s.pw[2 * p - 1], h);
+                }
             };
-            if (p == 0) {
-                T g[N + 1];
-                C::xrow(rowp, g);
-                C::yrest(g, h);
-            } else {
-                const T *r1 = r0 + S::kGrp;
-                auto rowm = [&](auto A) -> T {
+            if (edge)
+                sums([&](auto A) -> int {
                     constexpr int av = decltype(A)::value;
-                    return r1[av * SEG - e1<L1>(av)];
-                };
-                T gp[N + 1], gm[N + 1];
-                C::xrow(rowp, gp);
-                C::xrow(rowm, gm);
-                C::ypair_pw(gp, gm, s.pw[2 * p - 1], h);
-            }
+                    const int inside = tb + av * SEG - e1<L1>(av);
+                    const int l = (beyL >> av) & 1u ? S::kEnds + av : inside;
+                    return (beyR >> av) & 1u ? S::kEnds + Q1 + av : l;
+                });
+            else
+                sums([&](auto A) -> int { return tb + decltype(A)::value * SEG - e1<L1>(decltype(A)::value); });
             if (p == NP1) C::zfold_pw(h, s.pw[cz], R);
         }
         __syncwarp();  // every lane of this warp is done with buffer sb
@@ -888,8 +940,18 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
             for (int p = 1; p <= NP1; ++p) {
                 T Pp[N + 1], Pm[N + 1];
                 C::template yrows_pw<T>(Pc, s.pw[2 * p - 1], Pp, Pm);
-                C::emit_x(Pp, w3[p], cz * P2 + (2 * p - 1) * Q1, put);
-                C::emit_x(Pm, w3[p], cz * P2 + 2 * p * Q1, put);
+                if constexpr (std::is_same<T, float>::value) {  // both rows in packed pairs
+                    F2 Pr[N + 1];
+                    static_for<N + 1>([&](auto J) { Pr[decltype(J)::value] = F2(Pp[decltype(J)::value], Pm[decltype(J)::value]); });
+                    auto put2 = [&](int i, F2 v) {
+                        put(i, v.lo());
+                        put(i + Q1, v.hi());
+                    };
+                    TPCell<L1, N, F2>::emit_x(Pr, w3[p], cz * P2 + (2 * p - 1) * Q1, put2);
+                } else {
+                    C::emit_x(Pp, w3[p], cz * P2 + (2 * p - 1) * Q1, put);
+                    C::emit_x(Pm, w3[p], cz * P2 + 2 * p * Q1, put);
+                }
             }
         }
     }
