@@ -33,6 +33,7 @@ struct CtxView {
     int ntiles;
     const void *ghosts;
     const double *ghostsd;  // end-state deviations in double
+    long long *ghostsq;     // ... and in fixed point (D3Q39, D3Q103)
     unsigned *health;
     long long ncells;
     unsigned step;   // launch counter of lb_step (seeds the stochastic rounding)
@@ -83,6 +84,7 @@ StepArgs<Lat, T> make_args(const CtxView &v, const void *fin, void *fout) {
     a.tiles = v.tiles;
     a.ghosts = static_cast<const T *>(v.ghosts);
     a.ghostsd = v.ghostsd;
+    a.ghostsq = v.ghostsq;
     a.health = v.health;
     for (int i = 0; i < Lat::Q; ++i) a.plane[i] = v.plane[i];
     for (int p = 0; p <= Lat::NP; ++p) {
@@ -282,7 +284,7 @@ cudaError_t launch_ghost(const CtxView &v, const double *states, int ninst, void
     const StepArgs<Lat, T> a = make_args<Lat, T>(v, nullptr, nullptr);
     const int n = 2 * ninst;
     ghost_kernel<Lat, N, T><<<(n + 63) / 64, 64, 0, v.stream>>>(a, states, ninst, static_cast<T *>(ghosts),
-                                                                 ghostsd);
+                                                                 ghostsd, v.ghostsq);
     return cudaGetLastError();
 }
 

@@ -65,6 +65,7 @@ struct StepArgs {
     const int2 *__restrict__ tiles;  // line kernel: (instance, first x) per block
     const T *__restrict__ ghosts;    // [instance][2][Q], library order
     const double *__restrict__ ghostsd;  // the same end-state deviations in double
+    const long long *__restrict__ ghostsq;  // ... and in fixed point (split precision)
     unsigned *health;
     long long plane[Lat::Q];  // element offset of each population plane, library order
     T wp[Lat::NP + 1];        // weight of the rest velocity, then of each pair
@@ -289,6 +290,22 @@ struct Collide {
     static constexpr int KT = ntau(N);
     static constexpr SignOrbits<Lat> kOrb = SignOrbits<Lat>();
     static constexpr OrbitRows<Lat> kRows = OrbitRows<Lat>();
+    // f(row) for the orbits of one axis set: a loop over the run-time rows, or unrolled with
+    // compile-time ones on D3Q39, whose unrolled step fits the instruction caches (nine shocks of
+    // 108-325 cells: 17.4 us per step, 18.0 as loops)
+    template <int mask, class F>
+    SMRT_D static void for_rows(F &&f) {
+        constexpr int o0 = kRows.first[mask], o1 = kRows.first[mask + 1];
+        if constexpr (NP <= 19) {
+            static_for<o1 - o0>([&](auto O) {
+                constexpr typename OrbitRows<Lat>::Row r = kRows.row[o0 + decltype(O)::value];
+                f(r);
+            });
+        } else {
+#pragma unroll 1
+            for (int o = o0; o < o1; ++o) f(orbit_rows<Lat>().row[o]);
+        }
+    }
 
     // a2: conserved sums, in Acc. The state holds deviations df_i = f_i - w_i; the quadrature
     // gives sum w_i = 1, sum w_i xi_i = 0, sum w_i |xi_i|^2 = 3, so
@@ -413,10 +430,7 @@ struct Collide {
             constexpr int mask = decltype(Mk)::value + 1;
             constexpr int np = 1 << (mask_axes(mask) - 1);
             if constexpr (kRows.count(mask) > 0) {
-                constexpr int o0 = kRows.first[mask], o1 = kRows.first[mask + 1];
-#pragma unroll 1
-                for (int o = o0; o < o1; ++o) {
-                    const typename OrbitRows<Lat>::Row &r = orbit_rows<Lat>().row[o];
+                for_rows<mask>([&](const typename OrbitRows<Lat>::Row &r) {
                     long long S[np], D[np];
                     static_for<np>([&](auto B) {
                         constexpr int b = decltype(B)::value;
@@ -438,7 +452,7 @@ struct Collide {
                                 acc[g].madd(D[cl], r.mono[g]);
                         }
                     });
-                }
+                });
             }
         });
         static_for<Mm>([&](auto G) { R[decltype(G)::value] = acc[decltype(G)::value].value(); });
@@ -641,7 +655,7 @@ struct Collide {
     }
 
     // Split precision (T float): pullq(i, e, s, off) gives pulled population i, of vector s e, in
-    // fixed point (the stored float exactly, or the exact double end-state value beyond a fixed end),
+    // fixed point (the stored float exactly, or the double end-state value beyond a fixed end),
     // read once; store(i, value) receives post-collision population i as soon as it is formed.
     //
     // Code size. Unrolled over every population the D3Q103 step was 275 KB of instructions, far
@@ -842,10 +856,7 @@ struct Collide {
             constexpr int mask = decltype(Mk)::value + 1;
             constexpr int np = 1 << (mask_axes(mask) - 1);
             if constexpr (kRows.count(mask) > 0) {
-                constexpr int o0 = kRows.first[mask], o1 = kRows.first[mask + 1];
-#pragma unroll 1
-                for (int o = o0; o < o1; ++o) {
-                    const typename OrbitRows<Lat>::Row &r = orbit_rows<Lat>().row[o];
+                for_rows<mask>([&](const typename OrbitRows<Lat>::Row &r) {
                     SplitAcc Ea[np], Oa[np];
                     static_for<M>([&](auto G_) {
                         constexpr int g = decltype(G_)::value;
@@ -871,7 +882,7 @@ struct Collide {
                         out(r.ip[b], E[b] + Od[b]);
                         out(r.im[b], E[b] - Od[b]);
                     });
-                }
+                });
             }
         });
         return ok;
@@ -1020,8 +1031,7 @@ SMRT_D void line_tile(const StepArgs<Lat, T> &a, const T *__restrict__ fin, T *_
     const long long base = in.cell_off;
     const T *gl = a.ghosts + (long long)tile.x * 2 * Lat::Q;
     const T *gr = gl + Lat::Q;
-    const double *gld = a.ghostsd + (long long)tile.x * 2 * Lat::Q;
-    const double *grd = gld + Lat::Q;
+    const long long *glq = a.ghostsq + (long long)tile.x * 2 * Lat::Q;
     // pull of population i from cell xs of the instance: the stored state inside, the end
     // states beyond a fixed end
     auto pull = [&](int i, int xs) -> T {
@@ -1040,13 +1050,17 @@ SMRT_D void line_tile(const StepArgs<Lat, T> &a, const T *__restrict__ fin, T *_
         ok = C::collide_split(
             [&](int i, const signed char *e, int s, int) -> long long {
                 const int xs = x - (s * e[0] + in.kx);
-                if constexpr (FixedX) {
-                    if (xs < 0) return to_fixed(gld[i]);
-                    if (xs >= L) return to_fixed(grd[i]);
+                if constexpr (FixedX) {  // no branch: a cell inside the line, then the end state
+                    const bool lo = xs < 0, hi = xs >= L;
+                    const float v = load_pop<Coherent>(fin + a.plane[i] + base + (lo ? 0 : (hi ? L - 1 : xs)));
+                    probe = lo || hi ? probe : __fmaf_rn(v, 0.f, probe);
+                    const long long gq = glq[lo ? i : Lat::Q + i];
+                    return lo || hi ? gq : to_fixed(v);
+                } else {
+                    const float v = float(pull(i, xs));
+                    probe = __fmaf_rn(v, 0.f, probe);
+                    return to_fixed(v);
                 }
-                const float v = float(pull(i, xs));
-                probe = __fmaf_rn(v, 0.f, probe);
-                return to_fixed(v);
             },
             [&](int i, T v) { fout[a.plane[i] + base + x] = v; }, a.wsh, a.wsl, a.c, a.clo, tau_a<T>(in), tau_b<T>(in),
             mix32(unsigned(base + x) ^ mix32(step)), in.model, T(in.es_b));
@@ -1183,8 +1197,7 @@ SMRT_D bool line_warp_staged(const StepArgs<Lat, float> &a, const float *__restr
     parity ^= 1u;
     const int x = xw + lane;
     if (x >= L) return true;
-    const double *gld = a.ghostsd + (long long)tile.x * 2 * Lat::Q;
-    const double *grd = gld + Lat::Q;
+    const long long *glq = a.ghostsq + (long long)tile.x * 2 * Lat::Q;
     const int tb = int(base + x - in.kx - g_al);  // staged offset of this lane's pull with e_x = 0
     // does every pull of the warp's cells stay inside the line (warp-uniform)?
     const int xlast = (xw + 31 < L ? xw + 31 : L - 1);
@@ -1194,8 +1207,16 @@ SMRT_D bool line_warp_staged(const StepArgs<Lat, float> &a, const float *__restr
         float v = buf[tb + off];
         if (!inside) {
             const int xs = x - s * e[0] - in.kx;
-            if (xs < 0 || xs >= L) {
-                if constexpr (FixedX) return to_fixed(xs < 0 ? gld[i] : grd[i]);
+            const bool lo = xs < 0, hi = xs >= L;
+            if constexpr (FixedX) {
+                // the end states, in fixed point already, by selection: the pulls of an orbit stay in
+                // flight together (a diverged branch per pull, with a conversion on the
+                // double-precision pipe, made an edge warp the slowest of its block)
+                const long long gq = glq[lo ? i : Lat::Q + i];
+                v = lo || hi ? 0.f : v;
+                probe = __fmaf_rn(v, 0.f, probe);
+                return lo || hi ? gq : to_fixed(v);
+            } else if (lo || hi) {
                 v = load_pop<Coherent>(fin + a.plane[i] + base + wrap(xs, L));
             }
         }
@@ -1441,7 +1462,7 @@ __global__ void __launch_bounds__(128) fill_kernel(StepArgs<Lat, T> a, const dou
 // End-state populations of instance j: states[j] = (rho, u_phys, theta) left then right.
 template <class Lat, int N, class T>
 __global__ void ghost_kernel(StepArgs<Lat, T> a, const double *states, int ninst, T *ghosts,
-                             double *ghostsd) {
+                             double *ghostsd, long long *ghostsq) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 2 * ninst) return;
     const int j = t / 2;
@@ -1454,6 +1475,7 @@ __global__ void ghost_kernel(StepArgs<Lat, T> a, const double *states, int ninst
         constexpr int i = decltype(I)::value;
         ghosts[(long long)t * Lat::Q + i] = T(out[i]);
         ghostsd[(long long)t * Lat::Q + i] = out[i];
+        ghostsq[(long long)t * Lat::Q + i] = to_fixed(out[i]);
     });
 }
 
