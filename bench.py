@@ -367,7 +367,7 @@ def run_batched(args, world: int, rank: int, local: int) -> None:
     achieved = 2.0 * q * 4 * cells * K / (ms * 1e-3) / 1e9
     # the FP64 pipe bounds this kernel: its double-precision operations per cell-step (ncu
     # instruction counts, an FMA counted as two) against the nominal FP64 rate
-    # the kernel is bound by instruction issue (ncu: 26 % issue-active, instruction-fetch stalls
+    # the kernel is bound by instruction issue (ncu: 47 % issue-active, instruction-fetch stalls
     # first): its warp instructions per cell-step against one per clock per scheduler
     ginst = BATCHED_WARP_INST_PER_CELL * cells * K / (ms * 1e-3) / 1e9
     if rank != 0:
@@ -403,10 +403,9 @@ def run_batched(args, world: int, rank: int, local: int) -> None:
 TP_FP64_FLOP_PER_CELL = 14949.0
 FP64_PEAK_GFLOPS = 1250.0
 # warp instructions per cell-step of the split-precision D3Q103, N = 4 staged line kernel on the
-# 64 batched shocks (ncu smsp__inst_executed.sum of one launch / cells: 499.9 for the persistent
-# form, 501.9 for one plain launch per step), and the issue rate of a GB300 (4 schedulers per SM,
+# 64 batched shocks (ncu smsp__inst_executed.sum of one plain launch / cells), and the issue rate of a GB300 (4 schedulers per SM,
 # 152 SMs, 2070 MHz, one warp instruction per clock each)
-BATCHED_WARP_INST_PER_CELL = 499.9
+BATCHED_WARP_INST_PER_CELL = 562.8
 ISSUE_PEAK_GINST = 4 * 152 * 2.07
 
 
