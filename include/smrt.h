@@ -183,9 +183,8 @@ lb_status lb_step(lb_ctx *ctx, void *f_a, void *f_b, int nsteps);
 /* Launch schedule of the 1D-line (batched) kernels. tile_width: cells per block (32, 64, 128;
  * on D3Q729 and D3Q4913 a block of tile_width / 32 warps steps a tile of tile_width cells whose
  * pulls it stages once for all its warps, one 32-cell row per warp -- lb_init_lattice sets 128
- * for LB_F32 (stepped in tiles of 64 cells instead, with the same bits, where that takes fewer
- * rounds of blocks and no schedule has been set), 32 (D3Q729) or 64 (D3Q4913) for LB_F64, 128 on
- * the other sets; on D3Q729 the value
+ * for LB_F32 (or 64, with the same bits, where that takes fewer rounds of blocks), 32 (D3Q729) or
+ * 64 (D3Q4913) for LB_F64, 128 on the other sets; on D3Q729 the value
  * 1 selects one block per cell -- its populations in shared memory, the factored sums spread
  * over the block -- which lb_init_lattice picks for problems of at most 48 (LB_F64) or 32 (LB_F32)
  * cells per SM, and
@@ -224,8 +223,9 @@ lb_status lb_get_schedule(const lb_ctx *ctx, lb_schedule *schedule);
 lb_status lb_autotune(lb_ctx *ctx, void *f_a, void *f_b, int trial_steps, lb_schedule *best);
 
 /* lb_step_graph -- lb_step of a 1D-line context as a replay of a CUDA graph holding one
- * persistent launch of nsteps steps (captured on first use for this (f_a, f_b, nsteps,
- * schedule) and cached in the context; capture needs no allocation of device memory). Same
+ * persistent launch of nsteps steps (captured on first use for this (f_a, f_b, nsteps) and
+ * launch shape -- grid, tile table, x-row sums -- and cached in the context; capture needs no
+ * allocation of device memory). Same
  * buffer convention as lb_step. Errors: as lb_step, LB_ERR_UNSUPPORTED (box, a D3Q729 context
  * on its one-cell-per-block schedule, or a persistent kernel that cannot be resident),
  * LB_ERR_CUDA. */

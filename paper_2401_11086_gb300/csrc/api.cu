@@ -69,7 +69,8 @@ struct lb_ctx {
     cudaStream_t capture_stream;
     const void *graph_fa, *graph_fb;
     int graph_steps;
-    lb_schedule graph_sched;
+    long long graph_grid;  // the captured launch: blocks, cells per tile, tiles, x-row sums
+    int graph_width, graph_tiles, graph_tensor_cores;
 };
 
 namespace {
@@ -386,6 +387,7 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
     if (line && tensor && prec == LB_F32 && v.tile_width == 128) {
         bwidth = float_block_width(c);
         v.tile_width = bwidth;
+        c->sched.tile_width = bwidth;
     }
     if (!tiles.empty())
         e = cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, v.stream);
@@ -740,11 +742,15 @@ extern "C" lb_status lb_step_graph(lb_ctx *c, void *fa, void *fb, int nsteps) {
     lb_status st = check_pair(c, fa, fb, nsteps);
     if (st == LB_OK) st = flush_tables(c);
     if (st != LB_OK) return st;
-    if (!c->view.line || persistent_grid(c) < 1) return LB_ERR_UNSUPPORTED;
+    if (!c->view.line) return LB_ERR_UNSUPPORTED;
+    const long long grid = persistent_grid(c);
+    if (grid < 1) return LB_ERR_UNSUPPORTED;
+    // the tile tables are rewritten in place when the width changes: a graph is replayed only while
+    // the launch that it holds is the one that would be captured now
+    const int tiles = c->kind >= 2 ? c->view.nbtiles : c->view.ntiles;
     const bool same = c->graph && c->graph_fa == fa && c->graph_fb == fb && c->graph_steps == nsteps &&
-                      c->graph_sched.tile_width == c->sched.tile_width &&
-                      c->graph_sched.blocks_per_sm == c->sched.blocks_per_sm &&
-                      c->graph_sched.tensor_cores == c->sched.tensor_cores;
+                      c->graph_grid == grid && c->graph_width == c->view.tile_width && c->graph_tiles == tiles &&
+                      c->graph_tensor_cores == c->view.tensor_cores;
     if (!same) {
         if (c->graph) {
             cudaGraphExecDestroy(c->graph);
@@ -774,7 +780,10 @@ extern "C" lb_status lb_step_graph(lb_ctx *c, void *fa, void *fb, int nsteps) {
         c->graph_fa = fa;
         c->graph_fb = fb;
         c->graph_steps = nsteps;
-        c->graph_sched = c->sched;
+        c->graph_grid = grid;
+        c->graph_width = c->view.tile_width;
+        c->graph_tiles = tiles;
+        c->graph_tensor_cores = c->view.tensor_cores;
     }
     return cuda_status(cudaGraphLaunch(c->graph, c->view.stream));
 }

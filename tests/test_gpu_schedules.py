@@ -1,0 +1,69 @@
+"""Launch schedules of 1D-line contexts: what a context runs by default, what lb_get_schedule says of
+it, and that changing the schedule between graph replays changes nothing but the launch."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2401_11086_gb300 as P  # noqa: E402
+from paper_2401_11086_gb300 import shocks  # noqa: E402
+
+
+def _float_shocks(name, lengths):
+    d = P.lb_lattice_named(name)
+    Ma, theta1 = (3.0, 0.333) if name == "D3Q729" else (7.0, 0.071)
+    n = len(lengths)
+    ctx, f, _ = shocks.setup_batch(d, 5, [Ma] * n, lengths, precision="f32", width=0.0, theta1=[theta1] * n)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    f *= 1.0 + 1e-3 * torch.randn(f.shape, dtype=f.dtype, device="cuda", generator=g)
+    return ctx, f
+
+
+# more than 32 cells per SM on 152 SMs, below which D3Q729 takes one block per cell
+BATCHES = [[128] * 40, [1, 63, 64, 65, 127, 129, 200] * 8, [400] * 20]
+
+
+@pytest.mark.parametrize("name", ["D3Q729", "D3Q4913"])
+@pytest.mark.parametrize("lengths", BATCHES)
+@pytest.mark.parametrize("first,then", [(None, 128), (None, 64), (128, 64), (64, 32)])
+def test_graph_follows_a_change_of_tile_width(name, lengths, first, then):
+    """lb_step_graph under one width (None: the default), then under another, on the same buffers and
+    step count: bit for bit the persistent steps that the graphs hold."""
+    ctx, f = _float_shocks(name, lengths)
+    default = P.lb_get_schedule(ctx)["tile_width"]
+    if first is not None or default == 1:  # one block per cell has no graph form
+        P.lb_set_schedule(ctx, first or 64, 0, 0)
+    fa, fb = f.clone(), ctx.new_state()
+    P.lb_step_graph(ctx, fa, fb, 2)
+    P.lb_set_schedule(ctx, then, 0, 0)
+    P.lb_step_graph(ctx, fa, fb, 2)
+    ga, gb = f.clone(), ctx.new_state()
+    for width in (first or (64 if default == 1 else default), then):
+        P.lb_set_schedule(ctx, width, 0, 1)
+        P.lb_step(ctx, ga, gb, 2)
+    assert P.lb_poll_status(ctx)[0] == 0
+    assert torch.equal(ctx.planes(fa), ctx.planes(ga)) and torch.equal(ctx.planes(fb), ctx.planes(gb))
+
+
+def test_reported_width_is_the_one_that_runs():
+    """Float D3Q729 batches on both sides of the width rule, ragged ones among them, all above the size of
+    one block per cell: lb_get_schedule names the default width, 64 and 128 both occur, and setting the
+    reported schedule, or the other width, gives the default's bits."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cells = 32 * sms + 1
+    ragged = [1, 7, 63, 64, 65, 127, 128, 129]
+    batches = [[128] * (cells // 128 + 2), ragged * (cells // sum(ragged) + 1), [128] * sms, [1000] * sms]
+    seen = set()
+    for lengths in batches:
+        ctx, f = _float_shocks("D3Q729", lengths)
+        s = P.lb_get_schedule(ctx)
+        assert s["tile_width"] in (64, 128) and s["persistent"] == 0
+        seen.add(s["tile_width"])
+        want = ctx.planes(P.lb_step(ctx, f, ctx.new_state(), 1)).clone()
+        for width in (s["tile_width"], 192 - s["tile_width"]):
+            P.lb_set_schedule(ctx, width, s["blocks_per_sm"], s["persistent"], s["tensor_cores"])
+            assert torch.equal(ctx.planes(P.lb_step(ctx, f, ctx.new_state(), 1)), want)
+    assert seen == {64, 128}
