@@ -187,10 +187,10 @@ lb_status lb_step(lb_ctx *ctx, void *f_a, void *f_b, int nsteps);
  * 64 (D3Q4913) for LB_F64, 128 on the other sets; on D3Q729 the value
  * 1 selects one block per cell -- its populations in shared memory, the factored sums spread
  * over the block -- which lb_init_lattice picks for problems of at most 48 (LB_F64) or 32 (LB_F32)
- * cells per SM, and
- * which runs one launch per step only; on D3Q39 and D3Q103 an LB_F64 context of at most 32 cells
- * per SM that no schedule has been set on steps with a group of 16 or 32 threads per cell, which
- * sums in another order than one thread per cell: equal to round-off, not bit for bit);
+ * cells per SM; on D3Q39 and D3Q103 LB_F64 lines of at most 32 cells per SM the value 1, which
+ * lb_init_lattice picks for them, selects a group of 16 or 32 threads per cell, which sums in
+ * another order than one thread per cell: equal to round-off, not bit for bit; the value 1 runs
+ * one launch per step only);
  * persistent = 1: lb_step runs all its steps in one cooperative launch of blocks_per_sm
  * blocks per SM (0 = as many as fit), tiles spread over the blocks, a grid-wide barrier between
  * steps (its wait is bounded: on timeout the health word gets LB_HEALTH_TIMEOUT and the
@@ -209,13 +209,14 @@ typedef struct {
 } lb_schedule;
 
 /* lb_set_schedule / lb_get_schedule -- apply or read a schedule (a periodic box accepts only
- * {128, 0, 0, 0}). Setting a new tile width rebuilds the context's tile table (synchronises).
- * Errors: LB_ERR_INVALID, LB_ERR_UNSUPPORTED (persistent kernel cannot be resident; tensor_cores
- * on any other context), LB_ERR_CUDA. */
+ * {128, 0, 0, 0}). lb_get_schedule returns the schedule in effect, lb_init_lattice's choice until
+ * one is set; setting what it returns changes nothing. Setting a new tile width rebuilds the
+ * context's tile table (synchronises). Errors: LB_ERR_INVALID, LB_ERR_UNSUPPORTED (persistent
+ * kernel cannot be resident; tensor_cores, or tile width 1, on any other context), LB_ERR_CUDA. */
 lb_status lb_set_schedule(lb_ctx *ctx, const lb_schedule *schedule);
 lb_status lb_get_schedule(const lb_ctx *ctx, lb_schedule *schedule);
 
-/* lb_autotune -- time every candidate schedule (tile widths 32/64/128, and 1 on D3Q729; one
+/* lb_autotune -- time every candidate schedule (tile widths 32/64/128, and 1 where allowed; one
  * launch per step or persistent with 1, 2, 4 or all resident blocks per SM; x-row sums on the
  * CUDA cores and, where allowed, the tensor cores) for trial_steps steps on the states
  * f_a / f_b (which it ADVANCES: pass copies), apply the fastest and return it in *best with
@@ -226,7 +227,9 @@ lb_status lb_autotune(lb_ctx *ctx, void *f_a, void *f_b, int trial_steps, lb_sch
  * persistent launch of nsteps steps (captured on first use for this (f_a, f_b, nsteps) and
  * launch shape -- grid, tile table, x-row sums -- and cached in the context; capture needs no
  * allocation of device memory). Same
- * buffer convention as lb_step. Errors: as lb_step, LB_ERR_UNSUPPORTED (box, a D3Q729 context
+ * buffer convention as lb_step. On D3Q39 and D3Q103 at tile width 1 (groups of threads per cell,
+ * which have no persistent form) the graph steps one thread per cell in 128-cell tiles, equal to
+ * lb_step's results to round-off. Errors: as lb_step, LB_ERR_UNSUPPORTED (box, a D3Q729 context
  * on its one-cell-per-block schedule, or a persistent kernel that cannot be resident),
  * LB_ERR_CUDA. */
 lb_status lb_step_graph(lb_ctx *ctx, void *f_a, void *f_b, int nsteps);

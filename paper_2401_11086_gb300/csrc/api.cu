@@ -169,6 +169,12 @@ int float_block_width(const lb_ctx *c) {
     return rounds[1] < rounds[0] ? 64 : 128;
 }
 
+// Double lines on D3Q39 / D3Q103 small enough for groups of lanes (schedule tile width 1).
+bool lanes_allowed(const lb_ctx *c) {
+    return c->view.line && c->kind < 2 && c->prec == LB_F64 &&
+           c->view.ncells <= (long long)kLaneCellsPerSM * c->num_sms;
+}
+
 lb_status cuda_status(cudaError_t e) { return e == cudaSuccess ? LB_OK : LB_ERR_CUDA; }
 
 void free_tables(lb_ctx *c) {
@@ -369,8 +375,10 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
         e = cudaMalloc(&c->d_partials,
                        sizeof(double) * kMaxTau *
                            std::max(1LL, line ? std::max(c->max_tiles, lane_size ? kLaneMaxBlocks : 0) : adj_blocks(v)));
-    // small double lines step on groups of lanes until a schedule is set
-    v.lanes = line && !tensor && prec == LB_F64 && (long long)ncells <= (long long)kLaneCellsPerSM * c->num_sms;
+    if (e == cudaSuccess && lanes_allowed(c)) {
+        c->sched.tile_width = 1;
+        v.lanes = 1;
+    }
     // D3Q729 problems of at most 48 (double) or 32 (float) cells per SM take one block per cell
     // (measured crossovers with the tiled kernel)
     if (e == cudaSuccess && c->kind == 2 && (long long)ncells <= (prec == LB_F64 ? 48LL : 32LL) * c->num_sms) {
@@ -614,9 +622,10 @@ extern "C" lb_status lb_step(lb_ctx *c, void *fa, void *fb, int nsteps) {
 
 extern "C" lb_status lb_set_schedule(lb_ctx *c, const lb_schedule *s) {
     if (!c || !s) return LB_ERR_INVALID;
-    const bool cell_blocks = s->tile_width == 1;  // D3Q729: one cell per block, one launch per step
+    // one launch per step; D3Q729: one cell per block, D3Q39 / D3Q103: one per group of lanes
+    const bool cell_blocks = s->tile_width == 1;
     if (s->tile_width != 32 && s->tile_width != 64 && s->tile_width != 128 && !cell_blocks) return LB_ERR_INVALID;
-    if (cell_blocks && (c->kind != 2 || s->persistent)) return LB_ERR_UNSUPPORTED;
+    if (cell_blocks && ((c->kind != 2 && !lanes_allowed(c)) || s->persistent)) return LB_ERR_UNSUPPORTED;
     if (s->blocks_per_sm < 0 || (s->persistent != 0 && s->persistent != 1)) return LB_ERR_INVALID;
     if (s->tensor_cores != 0 && s->tensor_cores != 1) return LB_ERR_INVALID;
     // tensor-core x-rows: the block-staged kernels of float tensor-product lines with fixed ends
@@ -640,19 +649,20 @@ extern "C" lb_status lb_set_schedule(lb_ctx *c, const lb_schedule *s) {
             c->btile_width = s->tile_width;
         }
         c->view.tile_width = s->tile_width;
-    } else if (s->tile_width != c->view.tile_width) {
-        const std::vector<int2> tiles = make_tiles(c->nx_inst, s->tile_width);
+    } else if (const int width = cell_blocks ? kTile : s->tile_width; width != c->view.tile_width) {
+        // (the tiles that a context on groups of lanes starts with serve its other calls)
+        const std::vector<int2> tiles = make_tiles(c->nx_inst, width);
         if ((long long)tiles.size() > c->max_tiles) return LB_ERR_INVALID;
         cudaError_t e = cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(int2) * tiles.size(),
                                         cudaMemcpyHostToDevice, c->view.stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->view.stream);
         if (e != cudaSuccess) return LB_ERR_CUDA;
         c->view.ntiles = (int)tiles.size();
-        c->view.tile_width = s->tile_width;
+        c->view.tile_width = width;
     }
     c->sched = *s;
     c->view.tensor_cores = s->tensor_cores;
-    c->view.lanes = 0;
+    c->view.lanes = cell_blocks && c->kind < 2;
     if (c->sched.persistent && c->ks->occupancy(c->view) < 1) {
         c->sched.persistent = 0;
         return LB_ERR_UNSUPPORTED;
@@ -671,7 +681,7 @@ extern "C" lb_status lb_autotune(lb_ctx *c, void *fa, void *fb, int trial_steps,
     if (st != LB_OK || trial_steps < 1 || !best) return st != LB_OK ? st : LB_ERR_INVALID;
     std::vector<lb_schedule> cand;
     const int widths[4] = {32, 64, 128, 1};
-    const int nwidths = c->view.line ? (c->kind == 2 ? 4 : 3) : 1;
+    const int nwidths = c->view.line ? (c->kind == 2 || lanes_allowed(c) ? 4 : 3) : 1;
     // x-row sums on the CUDA cores, and on the tensor cores where the context allows it
     const int ntc = (c->kind >= 2 && c->prec == LB_F32 && c->view.line && c->view.fixedx) ? 2 : 1;
     for (int tc = 0; tc < ntc; ++tc)

@@ -51,7 +51,7 @@ struct CtxView {
     const int2 *btiles;
     int nbtiles;
     int num_sms;
-    int lanes;  // 1: the step of a small double line context runs on groups of lanes (lane_fits)
+    int lanes;  // 1: the step of a small double line context runs on groups of lanes (tile width 1)
 };
 
 using StepFn = cudaError_t (*)(const CtxView &, const void *fin, void *fout);

@@ -10,6 +10,7 @@ if not torch.cuda.is_available():
 
 import paper_2401_11086_gb300 as P  # noqa: E402
 from paper_2401_11086_gb300 import shocks  # noqa: E402
+from paper_2401_11086_gb300.autotune import tuned_schedule  # noqa: E402
 
 
 def _float_shocks(name, lengths):
@@ -67,3 +68,60 @@ def test_reported_width_is_the_one_that_runs():
             P.lb_set_schedule(ctx, width, s["blocks_per_sm"], s["persistent"], s["tensor_cores"])
             assert torch.equal(ctx.planes(P.lb_step(ctx, f, ctx.new_state(), 1)), want)
     assert seen == {64, 128}
+
+
+# ------------------------------------------------------------------ groups of lanes (tile width 1)
+LANES = [("D3Q39", 3, 1.25), ("D3Q103", 4, 2.0)]
+
+
+def _shocks(name, N, Ma, lengths, precision="f64"):
+    ctx, f, _ = shocks.setup_batch(P.lb_lattice_named(name), N, [Ma] * len(lengths), lengths, precision=precision,
+                                   width=4.0)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    f *= 1.0 + 1e-3 * torch.randn(f.shape, dtype=f.dtype, device="cuda", generator=g)
+    return ctx, f
+
+
+@pytest.mark.parametrize("name,N,Ma", LANES)
+@pytest.mark.parametrize("lengths", [[400], [130, 7, 300]])
+def test_small_double_lines_keep_their_default_schedule(name, N, Ma, lengths, tmp_path):
+    """The schedule that a small double line context starts on is reported, set again after others, chosen
+    by the autotuner (by more than a factor of two at these sizes) and stored, with the same bits."""
+    ctx, f = _shocks(name, N, Ma, lengths)
+    step = lambda c, nsteps=3: c.planes(P.lb_step(c, f.clone(), c.new_state(), nsteps)).clone()  # noqa: E731
+    want = step(ctx)
+    s = P.lb_get_schedule(ctx)
+    assert (s["tile_width"], s["persistent"]) == (1, 0)
+    put = lambda q: P.lb_set_schedule(ctx, q["tile_width"], q["blocks_per_sm"], q["persistent"],  # noqa: E731
+                                      q["tensor_cores"])
+    put(s)
+    assert torch.equal(step(ctx), want)
+    P.lb_set_schedule(ctx, 32, 0, 1)
+    other = step(ctx)
+    assert not torch.equal(other, want) and ((other - want).abs().max() / want.abs().max()).item() < 1e-13
+    put(s)
+    assert torch.equal(step(ctx), want)
+    best = P.lb_autotune(ctx, f.clone(), ctx.new_state(), 20)
+    assert best["tile_width"] == 1 and P.lb_get_schedule(ctx)["tile_width"] == 1
+    assert torch.equal(step(ctx), want)
+    path = str(tmp_path / "sched.json")
+    P.lb_set_schedule(ctx, 64, 0, 0)
+    assert tuned_schedule(ctx, f, lengths, trial_steps=20, path=path)["tile_width"] == 1
+    again, _ = _shocks(name, N, Ma, lengths)
+    P.lb_set_schedule(again, 64, 0, 0)
+    tuned_schedule(again, f, lengths, trial_steps=20, path=path)  # from the file
+    assert torch.equal(step(again), want)
+    assert P.lb_poll_status(ctx)[0] == 0
+
+
+def test_width_one_is_refused_elsewhere():
+    """Tile width 1 stays unsupported for persistent launches, float states and grids above 32 cells per SM,
+    and a refused schedule leaves the context as it was."""
+    big = 32 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    for lengths, precision, persistent in (([400], "f64", 1), ([400], "f32", 0), ([400], "f32c64", 0),
+                                           ([big], "f64", 0)):
+        ctx, f = _shocks("D3Q39", 3, 1.25, lengths, precision)
+        before = P.lb_get_schedule(ctx)
+        with pytest.raises(P.SmrtError) as e:
+            P.lb_set_schedule(ctx, 1, 0, persistent)
+        assert e.value.status == 5 and P.lb_get_schedule(ctx) == before
