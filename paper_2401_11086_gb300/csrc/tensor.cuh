@@ -104,18 +104,10 @@ struct TPTables {
     T e[L1::Q1];
     T w[L1::Q1];
     T pw[L1::Q1][kPow];  // e_a^k: the y and z passes read them instead of forming them per cell
-    // w_a w_b w_c by the classes (rest, then each pair) of c, b, a: rounded once, read per x-row
-    static constexpr int K = L1::NP1 + 1;
-    T w3[K * K][K];
 };
 
 template <class L1, class T, class U, bool Planes>
 SMRT_D void tp_load_tables(const TPArgs<T> &a, TPTables<L1, U, Planes> &s) {
-    constexpr int K = TPTables<L1, U, Planes>::K;
-    for (int i = threadIdx.x; i < K * K * K; i += blockDim.x) {
-        const int c = i / (K * K), b = i / K % K, q = i % K;  // class p > 0: abscissae 2 p - 1, 2 p
-        s.w3[i / K][q] = U(a.w1[c ? 2 * c - 1 : 0] * a.w1[b ? 2 * b - 1 : 0] * a.w1[q ? 2 * q - 1 : 0]);
-    }
     if constexpr (Planes)
         for (int i = threadIdx.x; i < TPTables<L1, U>::Q; i += blockDim.x) s.plane[i] = a.plane_idx[i];
     if (threadIdx.x < L1::Q1) {
@@ -126,6 +118,28 @@ SMRT_D void tp_load_tables(const TPArgs<T> &a, TPTables<L1, U, Planes> &s) {
         for (int k = 0; k < TPTables<L1, U>::kPow; ++k, p *= ea) s.pw[threadIdx.x][k] = p;
     }
     __syncthreads();
+}
+
+// The step's tables: also the weights w_a w_b w_c by the classes (rest, then each pair) of c, b, a,
+// rounded once and read per x-row. One row per unordered pair (b, c): a row per ordered pair took
+// 5.8 KB on D1Q17-P1 in double, and the third two-warp block no longer fitted an SM (24 shocks of
+// 1000 cells, N = 5: 3.32 ms per step with two blocks, 2.45 with three).
+template <class L1, class T, bool Planes = true>
+struct TPStepTables : TPTables<L1, T, Planes> {
+    static constexpr int K = L1::NP1 + 1;
+    T w3[K * (K + 1) / 2][K];
+    SMRT_HD static constexpr int row(int b, int c) { return b > c ? b * (b + 1) / 2 + c : c * (c + 1) / 2 + b; }
+};
+
+template <class L1, class T, bool Planes>
+SMRT_D void tp_load_step_tables(const TPArgs<T> &a, TPStepTables<L1, T, Planes> &s) {
+    constexpr int K = TPStepTables<L1, T, Planes>::K;
+    for (int i = threadIdx.x; i < K * K * K; i += blockDim.x) {
+        const int c = i / (K * K), b = i / K % K, q = i % K;  // class p > 0: abscissae 2 p - 1, 2 p
+        if (b <= c)
+            s.w3[s.row(b, c)][q] = T(a.w1[c ? 2 * c - 1 : 0] * a.w1[b ? 2 * b - 1 : 0] * a.w1[q ? 2 * q - 1 : 0]);
+    }
+    tp_load_tables<L1>(a, static_cast<TPTables<L1, T, Planes> &>(s));  // ends with __syncthreads
 }
 
 // Two floats in one 64-bit register pair: one packed instruction (add / multiply / fused
@@ -597,6 +611,14 @@ struct TPBlockStage {
     static constexpr size_t kBytes = 128 + size_t(kStages) * kStage * sizeof(T);  // mbarriers, buffers
 };
 
+// An SM's shared memory: 228 KB, of which each block takes 1 KB beside its own.
+constexpr size_t kSharedPerSM = 228 * 1024, kSharedPerBlock = 1024;
+// The double D1Q17-P1 step, bound by the FP64 pipe that an SM's warps share, keeps three blocks of
+// its two-warp tiles resident (128: the kernels' own scalars).
+static_assert(3 * (TPBlockStage<D1Q17P1, double, 2>::kBytes + sizeof(TPStepTables<D1Q17P1, double, false>) + 128 +
+                   kSharedPerBlock) <= kSharedPerSM,
+              "three blocks fit an SM");
+
 // ------------------------------------------------------------------ x-row sums on tensor cores
 // The x-row sums of one stage, g_j = sum_a f_a e_a^j for each of the warp's 32 cells and the
 // stage's one or two x-rows, as one warp-wide matrix product: rows (x-row, cell), columns
@@ -711,7 +733,7 @@ struct TPTensorRows {
 // TC (float, one warp per block): the x-row sums of every stage on the tensor cores.
 // Ident: the caller's plane order is the library's (no plane table lookups on the stores).
 template <class L1, int N, class T, int W, bool FixedX, bool Coherent, bool TC = false, bool Ident = false>
-SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, const T *__restrict__ fin,
+SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPStepTables<L1, T, false> &s, const T *__restrict__ fin,
                           T *__restrict__ fout, int tile_index, T *buf, unsigned long long *full,
                           unsigned long long *empty, unsigned nt, const CUtensorMap *tm) {
     using C = TPCell<L1, N, T>;
@@ -923,23 +945,28 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
         const bool ok = C::collide_moments(R, T(a.cd), tau_a<T>(in), tau_b<T>(in), in.model, T(in.es_b));
         if (!ok) atomicOr(a.health, 1u);
         C::x_from_powers(R);
-        constexpr int S_K = NP1 + 1;
         T *dst = fout + base + x;
         auto put = [&](int i, T v) { dst[plane(i) * a.stride] = v; };
 #pragma unroll 1
         for (int cz = 0; cz < Q1; ++cz) {
             T Pc[N + 1][N + 1];
             C::template zplane_pw<T>(R, s.pw[cz], Pc);
-            const T(*w3)[S_K] = s.w3 + ((cz + 1) >> 1) * S_K;
+            const int zc = (cz + 1) >> 1;
             {
                 T Pb[N + 1];
                 static_for<N + 1>([&](auto J) { Pb[decltype(J)::value] = Pc[decltype(J)::value][0]; });
-                C::emit_x(Pb, w3[0], cz * P2, put);
+                C::emit_x(Pb, s.w3[s.row(0, zc)], cz * P2, put);
             }
+            // rows (p, zc): a running pointer, or the index, whichever the compiler makes less of (D1Q17-P1 in
+            // double, one round of tiles, index against pointer: N = 5 1590 / 1529 us, N = 4 1345 / 1384)
+            constexpr bool kIndexed = Q1 == 17 && N < 5;
+            const T(*wrow)[NP1 + 1] = s.w3 + s.row(1, zc);
 #pragma unroll 1
             for (int p = 1; p <= NP1; ++p) {
                 T Pp[N + 1], Pm[N + 1];
                 C::template yrows_pw<T>(Pc, s.pw[2 * p - 1], Pp, Pm);
+                const T(&w3)[NP1 + 1] = kIndexed ? s.w3[s.row(p, zc)] : *wrow;
+                wrow += p < zc ? 1 : p + 1;
                 if constexpr (std::is_same<T, float>::value) {  // both rows in packed pairs
                     F2 Pr[N + 1];
                     static_for<N + 1>([&](auto J) { Pr[decltype(J)::value] = F2(Pp[decltype(J)::value], Pm[decltype(J)::value]); });
@@ -947,10 +974,10 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPTables<L1, T, false> &s, c
                         put(i, v.lo());
                         put(i + Q1, v.hi());
                     };
-                    TPCell<L1, N, F2>::emit_x(Pr, w3[p], cz * P2 + (2 * p - 1) * Q1, put2);
+                    TPCell<L1, N, F2>::emit_x(Pr, w3, cz * P2 + (2 * p - 1) * Q1, put2);
                 } else {
-                    C::emit_x(Pp, w3[p], cz * P2 + (2 * p - 1) * Q1, put);
-                    C::emit_x(Pm, w3[p], cz * P2 + 2 * p * Q1, put);
+                    C::emit_x(Pp, w3, cz * P2 + (2 * p - 1) * Q1, put);
+                    C::emit_x(Pm, w3, cz * P2 + 2 * p * Q1, put);
                 }
             }
         }
@@ -987,12 +1014,12 @@ constexpr int kTPMinBlocks = std::is_same<T, float>::value && !TC ? 4 : 0;
 // is 128-byte aligned, as the boxes need).
 template <class L1, int N, class T, int W, bool FixedX, bool TC = false, bool Ident = false>
 __global__ void __launch_bounds__(128, kTPMinBlocks<T, TC>) tp_step_line_block(TPArgs<T> a, int ntiles, const __grid_constant__ TPMaps maps) {
-    __shared__ TPTables<L1, T, false> s;
+    __shared__ TPStepTables<L1, T, false> s;
     extern __shared__ __align__(128) unsigned char dyn[];
     unsigned long long *full, *empty;
     T *buf;
     tp_block_setup<L1, T, W>(dyn, full, empty, buf);
-    tp_load_tables<L1>(a, s);  // ends with __syncthreads
+    tp_load_step_tables<L1>(a, s);  // ends with __syncthreads
     const int t = blockIdx.x;
     if (t >= ntiles) return;
     const CUtensorMap *tm = (a.tma && (smem_addr(dyn) & 127u) == 0u) ? &maps.src : nullptr;
@@ -1004,14 +1031,14 @@ __global__ void __launch_bounds__(128, kTPMinBlocks<T, TC>) tp_step_line_block(T
 template <class L1, int N, class T, int W, bool FixedX, bool TC = false, bool Ident = false>
 __global__ void __launch_bounds__(128, kTPMinBlocks<T, TC>) tp_step_line_persistent_block(TPArgs<T> a, int nsteps, int ntiles,
                                                                      unsigned *barg, const __grid_constant__ TPMaps maps) {
-    __shared__ TPTables<L1, T, false> s;
+    __shared__ TPStepTables<L1, T, false> s;
     __shared__ int failed;
     extern __shared__ __align__(128) unsigned char dyn[];
     unsigned long long *full, *empty;
     T *buf;
     tp_block_setup<L1, T, W>(dyn, full, empty, buf);
     if (threadIdx.x == 0) failed = 0;
-    tp_load_tables<L1>(a, s);
+    tp_load_step_tables<L1>(a, s);
     unsigned gen = 0;
     if (threadIdx.x == 0) gen = atomicAdd(&barg[1], 0u);
     const unsigned step0 = __ldcg(&barg[2]);
@@ -1064,9 +1091,9 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<float> a) {
     using C = TPCell<L1, N, float>;
     using SH = TPCellShared<L1, N>;
     constexpr int Q1 = SH::Q1, P2 = SH::P2, Q = SH::Q, M = SH::M;
-    __shared__ TPTables<L1, float> s;
+    __shared__ TPStepTables<L1, float> s;
     __shared__ SH sh;
-    tp_load_tables<L1>(a, s);  // ends with __syncthreads
+    tp_load_step_tables<L1>(a, s);  // ends with __syncthreads
     const int tid = threadIdx.x;
     const int2 tile = a.tiles[blockIdx.x >> 5];
     const InstanceInfo &in = a.inst[tile.x];
@@ -1158,7 +1185,7 @@ __global__ void __launch_bounds__(128) tp_step_cell_kernel(TPArgs<float> a) {
             });
             Pb[j] = acc;
         });
-        C::emit_x(Pb, s.w3[((c + 1) >> 1) * (L1::NP1 + 1) + ((b + 1) >> 1)], row * Q1, put);
+        C::emit_x(Pb, s.w3[s.row((b + 1) >> 1, (c + 1) >> 1)], row * Q1, put);
     }
 }
 
