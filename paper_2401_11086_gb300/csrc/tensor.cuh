@@ -1003,17 +1003,21 @@ SMRT_D void tp_block_setup(unsigned char *dyn, unsigned long long *&full, unsign
     }
 }
 
-// Blocks of 128 threads per SM that the float step kernels leave registers for (128 each). Without it
-// they take 168 and three blocks fit: the persistent launch then needs a second, nearly empty
-// round for 572 tiles on 152 SMs.
-template <class T, bool TC>
-constexpr int kTPMinBlocks = std::is_same<T, float>::value && !TC ? 4 : 0;
+// Blocks of 128 threads per SM that the step kernels leave registers for (0: the compiler's own
+// choice). Float: 4 (128 registers) for lines with fixed ends on D1Q9-P1. Without it they take 168
+// and three blocks fit: the persistent launch then needs a second, nearly empty round for 572 tiles
+// on 152 SMs. Else 3 (168): on D1Q17-P1 three 128-cell blocks fill the shared memory, and the wrapped
+// pulls of a periodic line take more registers; 128 of them only made spills there. N = 5 (N = 4), ms
+// per step, 128 -> 168: 64 lines of 325 cells on D1Q17-P1 0.316 -> 0.275; 64 periodic lines of 400,
+// persistent, D1Q9-P1 0.232 -> 0.144 (0.211 -> 0.140), D1Q17-P1 1.92 -> 1.81 (1.85 -> 1.06).
+template <class L1, class T, bool FixedX, bool TC>
+constexpr int kTPMinBlocks = std::is_same<T, float>::value && !TC ? (FixedX && L1::Q1 == 9 ? 4 : 3) : 0;
 
 // One step: block b (W warps) takes the block tile b.
 // maps: tensor maps of the two states, used when a.tma is set (and the dynamic shared memory
 // is 128-byte aligned, as the boxes need).
 template <class L1, int N, class T, int W, bool FixedX, bool TC = false, bool Ident = false>
-__global__ void __launch_bounds__(128, kTPMinBlocks<T, TC>) tp_step_line_block(TPArgs<T> a, int ntiles, const __grid_constant__ TPMaps maps) {
+__global__ void __launch_bounds__(128, kTPMinBlocks<L1, T, FixedX, TC>) tp_step_line_block(TPArgs<T> a, int ntiles, const __grid_constant__ TPMaps maps) {
     __shared__ TPStepTables<L1, T, false> s;
     extern __shared__ __align__(128) unsigned char dyn[];
     unsigned long long *full, *empty;
@@ -1029,7 +1033,7 @@ __global__ void __launch_bounds__(128, kTPMinBlocks<T, TC>) tp_step_line_block(T
 // All nsteps steps in one cooperative launch (see step_line_persistent in kernels.cuh); the
 // blocks stride over the block tiles.
 template <class L1, int N, class T, int W, bool FixedX, bool TC = false, bool Ident = false>
-__global__ void __launch_bounds__(128, kTPMinBlocks<T, TC>) tp_step_line_persistent_block(TPArgs<T> a, int nsteps, int ntiles,
+__global__ void __launch_bounds__(128, kTPMinBlocks<L1, T, FixedX, TC>) tp_step_line_persistent_block(TPArgs<T> a, int nsteps, int ntiles,
                                                                      unsigned *barg, const __grid_constant__ TPMaps maps) {
     __shared__ TPStepTables<L1, T, false> s;
     __shared__ int failed;
