@@ -52,6 +52,7 @@ struct lb_ctx {
     // device tables owned by the context
     InstanceInfo *d_inst;
     int2 *d_tiles;
+    int2 *d_ltiles;      // groups of lanes: (instance, first x) of each block of the step
     int2 *d_btiles;      // tensor-product lines: block tiles of the step kernels (tile_width cells)
     int *d_plane;        // tensor-product sets: caller plane of each library population
     void *d_ghosts;
@@ -182,6 +183,7 @@ void free_tables(lb_ctx *c) {
     cudaFree(c->d_inst);
     cudaFree(c->d_tiles);
     cudaFree(c->d_btiles);
+    cudaFree(c->d_ltiles);
     cudaFree(c->d_plane);
     cudaFree(c->d_ghosts);
     cudaFree(c->d_ghostsd);
@@ -375,9 +377,13 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
         e = cudaMalloc(&c->d_partials,
                        sizeof(double) * kMaxTau *
                            std::max(1LL, line ? std::max(c->max_tiles, lane_size ? kLaneMaxBlocks : 0) : adj_blocks(v)));
+    std::vector<int2> ltiles;
     if (e == cudaSuccess && lanes_allowed(c)) {
         c->sched.tile_width = 1;
         v.lanes = 1;
+        ltiles = make_tiles(c->nx_inst, kLaneThreads / lane_group(v));
+        v.nltiles = (int)ltiles.size();
+        e = cudaMalloc(&c->d_ltiles, sizeof(int2) * ltiles.size());
     }
     // D3Q729 problems of at most 48 (double) or 32 (float) cells per SM take one block per cell
     // (measured crossovers with the tiled kernel)
@@ -399,6 +405,8 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
     }
     if (!tiles.empty())
         e = cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, v.stream);
+    if (e == cudaSuccess && !ltiles.empty())
+        e = cudaMemcpyAsync(c->d_ltiles, ltiles.data(), sizeof(int2) * ltiles.size(), cudaMemcpyHostToDevice, v.stream);
     // block tiles of the default width (a one-cell-per-block schedule leaves them unused until a
     // tiled width is set)
     const std::vector<int2> btiles = line && tensor ? make_tiles(c->nx_inst, bwidth) : std::vector<int2>();
@@ -426,6 +434,7 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
     v.inst = c->d_inst;
     v.tiles = c->d_tiles;
     v.btiles = c->d_btiles;
+    v.ltiles = c->d_ltiles;
     v.plane_idx = c->d_plane;
     v.ghosts = c->d_ghosts;
     v.ghostsd = c->d_ghostsd;

@@ -50,6 +50,9 @@ struct CtxView {
     // tensor-product lines: the step kernels' block tiles (instance, first x) of tile_width cells
     const int2 *btiles;
     int nbtiles;
+    // groups of lanes: (instance, first x) of each block of the step
+    const int2 *ltiles;
+    int nltiles;
     int num_sms;
     int lanes;  // 1: the step of a small double line context runs on groups of lanes (tile width 1)
 };
@@ -194,21 +197,26 @@ cudaError_t lane_smem_limit(size_t bytes) {
     return e;
 }
 
+// bpt blocks for each of the ntiles tiles of the arguments' table
 template <auto Kernel, class Sh, class... A>
-cudaError_t lane_launch(const CtxView &v, const A &...args) {
+cudaError_t lane_launch(const CtxView &v, int ntiles, int bpt, const A &...args) {
     const cudaError_t e = lane_smem_limit<Kernel>(sizeof(Sh));
     if (e != cudaSuccess) return e;
-    const int bpt = lane_blocks_per_tile(v);
-    Kernel<<<v.ntiles * bpt, kLaneThreads, sizeof(Sh), v.stream>>>(args..., bpt);
+    Kernel<<<ntiles * bpt, kLaneThreads, sizeof(Sh), v.stream>>>(args..., bpt);
     return cudaGetLastError();
 }
+// The step's blocks are listed one by one. Sixteen for each 128-cell tile were 9600 on 600 lines of
+// 8 cells, all but 600 without a cell, and slower than one thread per cell: D3Q39, N = 3, 49 us per
+// step against 35 (27 with 600 blocks); D3Q103, N = 4, 69 (49).
 template <class Lat, int N, bool FixedX, int G>
-cudaError_t lane_step(const CtxView &v, const StepArgs<Lat, double> &a) {
-    return lane_launch<step_lane_kernel<Lat, N, FixedX, G>, LaneShared<Lat, N, false, G>>(v, a);
+cudaError_t lane_step(const CtxView &v, StepArgs<Lat, double> a) {
+    a.tiles = v.ltiles;
+    return lane_launch<step_lane_kernel<Lat, N, FixedX, G>, LaneShared<Lat, N, false, G>>(v, v.nltiles, 1, a);
 }
 template <class Lat, int N, class T, bool FixedX, int G>
 cudaError_t lane_adjoint(const CtxView &v, const StepArgs<Lat, T> &a, const double *in, double *out, double *partials) {
-    return lane_launch<adjoint_lane_kernel<Lat, N, T, FixedX, G>, LaneShared<Lat, N, true, G>>(v, a, in, out, partials);
+    return lane_launch<adjoint_lane_kernel<Lat, N, T, FixedX, G>, LaneShared<Lat, N, true, G>>(
+        v, v.ntiles, lane_blocks_per_tile(v), a, in, out, partials);
 }
 
 template <class Lat, int N, class T, class Acc, bool Split>
