@@ -1207,8 +1207,8 @@ SMRT_D bool line_warp_staged(const StepArgs<Lat, float> &a, const float *__restr
         float v = buf[tb + off];
         if (!inside) {
             const int xs = x - s * e[0] - in.kx;
-            const bool lo = xs < 0, hi = xs >= L;
             if constexpr (FixedX) {
+                const bool lo = xs < 0, hi = xs >= L;
                 // the end states, in fixed point already, by selection: the pulls of an orbit stay in
                 // flight together (a diverged branch per pull, with a conversion on the
                 // double-precision pipe, made an edge warp the slowest of its block)
@@ -1216,7 +1216,9 @@ SMRT_D bool line_warp_staged(const StepArgs<Lat, float> &a, const float *__restr
                 v = lo || hi ? 0.f : v;
                 probe = __fmaf_rn(v, 0.f, probe);
                 return lo || hi ? gq : to_fixed(v);
-            } else if (lo || hi) {
+            } else {
+                // periodic: no branch either, every lane of an edge warp loads (4 lines of 512 cells, us
+                // per step, with a branch per pull: D3Q39 16.4 -> 12.4; D3Q103, N = 4 43.1 -> 41.0)
                 v = load_pop<Coherent>(fin + a.plane[i] + base + wrap(xs, L));
             }
         }
