@@ -192,7 +192,8 @@ lb_status lb_step(lb_ctx *ctx, void *f_a, void *f_b, int nsteps);
  * another order than one thread per cell: equal to round-off, not bit for bit; the value 1 runs
  * one launch per step only);
  * persistent = 1: lb_step runs all its steps in one cooperative launch of blocks_per_sm
- * blocks per SM (0 = as many as fit), tiles spread over the blocks, a grid-wide barrier between
+ * blocks per SM (0 = as many as fit, or fewer where that ends sooner), tiles spread over the blocks,
+ * a grid-wide barrier between
  * steps (its wait is bounded: on timeout the health word gets LB_HEALTH_TIMEOUT and the
  * launch ends); persistent = 0: one launch per step. tensor_cores = 1 (LB_F32 D3Q729 / D3Q4913
  * lines with fixed ends, tile width 32): the x-row sums of the projection (Eq. an, the

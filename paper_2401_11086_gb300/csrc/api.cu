@@ -591,7 +591,33 @@ lb_status check_pair(const lb_ctx *c, const void *fa, const void *fb, int nsteps
     return LB_OK;
 }
 
-// grid of the persistent launch: blocks_per_sm (0 = as many as fit) on every SM, at most one
+// Blocks per SM of a persistent launch that leaves them open, of the occ that fit. A block strides
+// over the tiles, so a step takes ceil(tiles / blocks) rounds, and the last one, with a tile for few
+// blocks, takes as long as a full one: those blocks share SMs. With few rounds, fewer blocks that
+// spread the tiles evenly end sooner:
+// - double tensor-product kernels are bound by the FP64 pipe that an SM's warps share: a round takes
+//   as long as it has blocks per SM, and at least as long as its warps take to fill the four
+//   sub-partitions. ms per step, N = 5, all that fit -> fewer: D3Q4913, 300 shocks of 100 cells (600
+//   tiles) 4.87 -> 3.37; D3Q729, 64 of 800, 32-cell tiles 1.21 -> 0.94, 128-cell tiles 1.21 -> 0.98.
+//   Above three rounds nothing is left to gain (512 shocks of 100-400 cells, six rounds: 3.63 -> 3.68);
+// - split precision (staged), two rounds: the fewest blocks that still take two. 64 shocks of 1000
+//   cells (512 tiles), us per step: D3Q103 N = 4 114 -> 99, N = 3 97 -> 85, D3Q39 42 -> 36.
+// Other kernels are bound by latency and run best with all that fit (the float D3Q103 shocks: 46 us
+// with three blocks per SM, 61 with two).
+int open_blocks(const lb_ctx *c, int occ, long long tiles) {
+    auto rounds = [&](int b) { return (tiles + (long long)b * c->num_sms - 1) / ((long long)b * c->num_sms); };
+    int best = occ;
+    if (c->kind >= 2 && c->prec == LB_F64 && rounds(occ) <= 3) {
+        const int fill = 128 / c->view.tile_width;
+        for (int b = occ - 1; b >= 1; --b)
+            if (rounds(b) * std::max(b, fill) < rounds(best) * std::max(best, fill)) best = b;
+    } else if (c->prec == LB_F32_CONS64 && c->view.plane_identity && rounds(occ) == 2) {
+        while (best > 1 && rounds(best - 1) == 2) --best;
+    }
+    return best;
+}
+
+// grid of the persistent launch: blocks_per_sm (0 = open_blocks) on every SM, at most one
 // block per tile
 long long persistent_grid(const lb_ctx *c) {
     // blocks with work: one per tile (block tiles on tensor-product sets, whose
@@ -599,8 +625,8 @@ long long persistent_grid(const lb_ctx *c) {
     if (c->kind >= 2 && c->view.tile_width < 32) return 0;
     const int occ = c->ks->occupancy(c->view);
     if (occ < 1) return 0;
-    const int bps = c->sched.blocks_per_sm > 0 ? std::min(c->sched.blocks_per_sm, occ) : occ;
     const long long needed = c->kind >= 2 ? c->view.nbtiles : c->view.ntiles;
+    const int bps = c->sched.blocks_per_sm > 0 ? std::min(c->sched.blocks_per_sm, occ) : open_blocks(c, occ, needed);
     return std::max(1LL, std::min((long long)bps * c->num_sms, needed));
 }
 

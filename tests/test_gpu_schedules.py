@@ -125,3 +125,26 @@ def test_width_one_is_refused_elsewhere():
         with pytest.raises(P.SmrtError) as e:
             P.lb_set_schedule(ctx, 1, 0, persistent)
         assert e.value.status == 5 and P.lb_get_schedule(ctx) == before
+
+
+# ------------------------------------------------------------------ blocks of the persistent launch
+@pytest.mark.parametrize("name,N,Ma,precision,cells", [("D3Q729", 4, 3.0, "f64", 20), ("D3Q4913", 5, 7.0, "f64", 40),
+                                                       ("D3Q103", 4, 2.0, "f32c64", 40), ("D3Q39", 3, 1.25, "f32c64", 40)])
+@pytest.mark.parametrize("per_sm", [1, 3.2, 6.5])
+def test_open_number_of_blocks_gives_the_same_bits(name, N, Ma, precision, cells, per_sm):
+    """The persistent launch that leaves its blocks open (blocks_per_sm 0), below, in and above the range where
+    it takes fewer than fit, against one block per SM: the same kernel on another grid."""
+    count = int(per_sm * torch.cuda.get_device_properties(0).multi_processor_count)
+    theta1 = {"D3Q729": [0.333] * count, "D3Q4913": [0.071] * count}.get(name)
+    ctx, f, _ = shocks.setup_batch(P.lb_lattice_named(name), N, [Ma] * count, [cells] * count, precision=precision,
+                                   width=0.0, theta1=theta1)
+    for width in (128, 64):
+        runs = []
+        for blocks in (0, 1):
+            P.lb_set_schedule(ctx, width, blocks, 1)
+            runs.append(ctx.planes(P.lb_step(ctx, f.clone(), ctx.new_state(), 3)).clone())
+            assert P.lb_poll_status(ctx)[0] == 0
+            if precision != "f64":  # the step counter seeds the stochastic rounding: start both alike
+                ctx, _, _ = shocks.setup_batch(P.lb_lattice_named(name), N, [Ma] * count, [cells] * count,
+                                               precision=precision, width=0.0, theta1=theta1)
+        assert torch.equal(runs[0], runs[1])
