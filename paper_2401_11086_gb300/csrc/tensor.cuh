@@ -959,7 +959,7 @@ SMRT_D bool tp_block_tile(const TPArgs<T> &a, const TPStepTables<L1, T, false> &
             }
             // rows (p, zc): a running pointer, or the index, whichever the compiler makes less of (D1Q17-P1 in
             // double, one round of tiles, index against pointer: N = 5 1590 / 1529 us, N = 4 1345 / 1384)
-            constexpr bool kIndexed = Q1 == 17 && N < 5;
+            constexpr bool kIndexed = N < 5;
             const T(*wrow)[NP1 + 1] = s.w3 + s.row(1, zc);
 #pragma unroll 1
             for (int p = 1; p <= NP1; ++p) {
