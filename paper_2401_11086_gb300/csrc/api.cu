@@ -146,12 +146,15 @@ int max_reach(int axis) {
     return m;
 }
 
-// Cells per block tile of a float tensor-product context until a schedule is set: 128, or 64 when
-// that takes fewer rounds of resident blocks, or, within one round, fewer cells (with the padding
-// of the lines' last tiles) on the fullest SM. The step gives the same bits either way. Measured on
-// D3Q729, N = 5, 152 SMs, us per step, 128 / 64 cells: 1216 tiles of 128 cells (two rounds either
-// way) 162 / 164; lines of 100-400 cells: 64 of them 49 / 43, 128 63 / 56, 256 148 / 105 (two
-// rounds / one), 384 162 / 169, 512 232 / 203 (three / two), 700 262 / 268.
+// Cells per block tile of a float tensor-product context until a schedule is set:
+// 128, or 64 when that takes fewer rounds of resident blocks, or, within one round, fewer cells (with
+// the padding of the lines' last tiles) on the fullest SM. The step gives the same bits either way.
+// Measured on 152 SMs, lines of 100-400 cells, us per step, 128 / 64 cells (* the rule's choice):
+//   D3Q729, N = 5     64 lines 51 / 43*, 256 142 / 107*, 384 156* / 165, 512 228 / 200*, 700 261* / 269
+//   D3Q4913, N = 5    8 lines 162 / 149*, 56 193* / 205, 64 252 / 219*, 96 307 / 298*, 160 496 / 505*,
+//                     200 718* / 688
+// Periodic lines on D3Q729 keep 128: their tiles' ends, rewritten in the staged rows, cost more the more
+// tiles there are (64 lines of 400 cells, N = 5, 139 / 161, persistent 144 / 168).
 int float_block_width(const lb_ctx *c) {
     long long rounds[2], load[2];
     for (int i = 0; i < 2; ++i) {
@@ -398,7 +401,7 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
         return e == cudaErrorMemoryAllocation ? LB_ERR_NOMEM : LB_ERR_CUDA;
     }
     int bwidth = width0;
-    if (line && tensor && prec == LB_F32 && v.tile_width == 128) {
+    if (line && tensor && prec == LB_F32 && (v.fixedx || c->kind == 3) && v.tile_width == 128) {
         bwidth = float_block_width(c);
         v.tile_width = bwidth;
         c->sched.tile_width = bwidth;

@@ -148,3 +148,24 @@ def test_open_number_of_blocks_gives_the_same_bits(name, N, Ma, precision, cells
                 ctx, _, _ = shocks.setup_batch(P.lb_lattice_named(name), N, [Ma] * count, [cells] * count,
                                                precision=precision, width=0.0, theta1=theta1)
         assert torch.equal(runs[0], runs[1])
+
+
+def test_periodic_float_lines_start_on_128_cell_tiles(name="D3Q729"):
+    """At sizes where lines with fixed ends start on 64-cell tiles; the bits of either width."""
+    d = P.lb_lattice_named(name)
+    lengths = [128] * (32 * torch.cuda.get_device_properties(0).multi_processor_count // 128 + 2)
+    assert P.lb_get_schedule(_float_shocks(name, lengths)[0])["tile_width"] == 64
+    ctx = P.lb_init_lattice(P.LatticeDesc(d.e, d.w, d.c, d.degree, (1, 0, 0)), 0, N=5, precision="f32",
+                            nx_per_instance=lengths)
+    assert P.lb_get_schedule(ctx)["tile_width"] == 128
+    P.lb_set_relaxation(ctx, [2.0] * shocks.ntau(5), True, 1.0)
+    one = torch.ones(ctx.cells, dtype=torch.float64, device="cuda")
+    f = ctx.new_state()
+    P.lb_fill_equilibrium(ctx, f, one, torch.stack([d.c * one, 0 * one, 0 * one]).contiguous(), one)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    f *= 1.0 + 1e-3 * torch.randn(f.shape, dtype=f.dtype, device="cuda", generator=g)
+    want = ctx.planes(P.lb_step(ctx, f, ctx.new_state(), 1)).clone()
+    for width in (128, 64):
+        P.lb_set_schedule(ctx, width, 0, 0)
+        assert torch.equal(ctx.planes(P.lb_step(ctx, f, ctx.new_state(), 1)), want)
+    assert P.lb_poll_status(ctx)[0] == 0
