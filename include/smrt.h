@@ -140,7 +140,8 @@ lb_status lb_set_relaxation(lb_ctx *ctx, const double *tau, int maxwell_molecule
  * lb_set_relaxation so that the end-state populations use the new frame (end states already set
  * are recomputed in the new frame). Stored on the host and uploaded as lb_set_relaxation's
  * settings are.
- * Errors: LB_ERR_INVALID (bad instance; a single box accepts only -1), LB_ERR_CUDA. */
+ * Errors: LB_ERR_INVALID (bad instance; a single box accepts only -1; on a periodic x axis, the
+ * set's reach plus |kx| above the length of an instance), LB_ERR_CUDA. */
 lb_status lb_set_frame_shift(lb_ctx *ctx, int instance, int kx);
 
 /* Collision models of lb_set_collision_model. */

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <map>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -33,6 +34,7 @@ using namespace smrt;
 struct lb_ctx {
     int kind;  // 0 D3Q39, 1 D3Q103, 2 D3Q729 (D1Q9-P1 cubed), 3 D3Q4913 (D1Q17-P1 cubed)
     int q, np, N, degree;
+    int reach;  // largest |e_x| of the set
     lb_precision prec;
     size_t elem;  // bytes per population value
     const KernelSet *ks;
@@ -266,6 +268,7 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
         }
     }
 
+    c->reach = reach[0];
     // geometry
     const bool line = (grid->ny == 1 && grid->nz == 1);
     c->batch = grid->batch;
@@ -549,6 +552,10 @@ extern "C" lb_status lb_set_frame_shift(lb_ctx *c, int instance, int kx) {
     if (!c || instance < -1 || instance >= c->batch) return LB_ERR_INVALID;
     if (!c->view.line && instance != -1) return LB_ERR_INVALID;
     const int j0 = instance < 0 ? 0 : instance, j1 = instance < 0 ? c->batch : instance + 1;
+    // a periodic x axis wraps at most once, as for the shift given to lb_init_lattice
+    if (!c->view.fixedx)
+        for (int j = j0; j < j1; ++j)
+            if (c->reach + std::llabs((long long)kx) > c->nx_inst[j]) return LB_ERR_INVALID;
     for (int j = j0; j < j1; ++j) c->h_inst[j].kx = kx;
     if (!c->view.line) c->view.kx = kx;
     if (c->relax_set)

@@ -1,5 +1,5 @@
 """1D lines at their ends and in numbers: many short lines on groups of lanes, wrapped pulls of periodic
-split-precision lines."""
+split-precision lines, and frame shifts that a periodic axis cannot hold."""
 import numpy as np
 import pytest
 
@@ -64,3 +64,26 @@ def test_periodic_split_lines_staged_and_direct(name, N, shift, persistent):
         got[torch.from_numpy(o).cuda()] = out
         res.append(got.double())
     assert ((res[0] - res[1]).abs().max() / res[1].abs().max()).item() < 3 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("name,N,precision", [("D3Q39", 3, "f64"), ("D3Q103", 4, "f32c64"), ("D3Q729", 4, "f32")])
+def test_frame_shift_beyond_a_periodic_line_is_refused(name, N, precision):
+    """Pulls wrap once: reach + |k_x| above the length of a periodic instance is refused by lb_set_frame_shift
+    as it is by lb_init_lattice, and nothing changes; the largest shift that fits, and any shift of a line
+    with fixed ends, are taken."""
+    d = P.lb_lattice_named(name)
+    reach = int(np.abs(d.e[:, 0]).max())
+    desc = P.LatticeDesc(d.e, d.w, d.c, d.degree, (0, 0, 0))
+    ctx = P.lb_init_lattice(desc, 0, N=N, precision=precision, nx_per_instance=[40, 20])
+    for instance, kx in ((1, 21 - reach), (1, reach - 21), (-1, 21 - reach), (0, 41 - reach), (0, -2 ** 31), (0, 2 ** 31 - 1)):
+        with pytest.raises(P.SmrtError) as e:
+            P.lb_set_frame_shift(ctx, instance, kx)
+        assert e.value.status == 1
+    P.lb_set_frame_shift(ctx, 1, 20 - reach)
+    P.lb_set_frame_shift(ctx, 0, reach - 40)
+    P.lb_set_frame_shift(P.lb_init_lattice(desc, 0, N=N, precision=precision, bc_x=1, nx_per_instance=[4]), 0, 50)
+    if name == "D3Q39":
+        box = P.lb_init_lattice(desc, 12, 9, 9, N=N, precision=precision)
+        P.lb_set_frame_shift(box, -1, 12 - reach)
+        with pytest.raises(P.SmrtError):
+            P.lb_set_frame_shift(box, -1, 13 - reach)
