@@ -32,8 +32,7 @@ struct CtxView {
     const int2 *tiles;
     int ntiles;
     const void *ghosts;
-    const double *ghostsd;  // end-state deviations in double
-    long long *ghostsq;     // ... and in fixed point (D3Q39, D3Q103)
+    long long *ghostsq;  // the end states in fixed point (D3Q39, D3Q103)
     unsigned *health;
     long long ncells;
     unsigned step;   // launch counter of lb_step (seeds the stochastic rounding)
@@ -61,8 +60,7 @@ using StepFn = cudaError_t (*)(const CtxView &, const void *fin, void *fout);
 using MomentsFn = cudaError_t (*)(const CtxView &, const void *f, double *out, unsigned mask);
 using FillFn = cudaError_t (*)(const CtxView &, void *f, const double *rho, const double *u,
                                const double *theta);
-using GhostFn = cudaError_t (*)(const CtxView &, const double *states, int ninst, void *ghosts,
-                                double *ghostsd);
+using GhostFn = cudaError_t (*)(const CtxView &, const double *states, int ninst, void *ghosts);
 
 using PersistFn = cudaError_t (*)(const CtxView &, void *fa, void *fb, int nsteps, int grid);
 using OccupancyFn = int (*)(const CtxView &);
@@ -86,7 +84,6 @@ StepArgs<Lat, T> make_args(const CtxView &v, const void *fin, void *fout) {
     a.inst = v.inst;
     a.tiles = v.tiles;
     a.ghosts = static_cast<const T *>(v.ghosts);
-    a.ghostsd = v.ghostsd;
     a.ghostsq = v.ghostsq;
     a.health = v.health;
     for (int i = 0; i < Lat::Q; ++i) a.plane[i] = v.plane[i];
@@ -288,11 +285,11 @@ cudaError_t launch_fill(const CtxView &v, void *f, const double *rho, const doub
 }
 
 template <class Lat, int N, class T>
-cudaError_t launch_ghost(const CtxView &v, const double *states, int ninst, void *ghosts, double *ghostsd) {
+cudaError_t launch_ghost(const CtxView &v, const double *states, int ninst, void *ghosts) {
     const StepArgs<Lat, T> a = make_args<Lat, T>(v, nullptr, nullptr);
     const int n = 2 * ninst;
     ghost_kernel<Lat, N, T><<<(n + 63) / 64, 64, 0, v.stream>>>(a, states, ninst, static_cast<T *>(ghosts),
-                                                                 ghostsd, v.ghostsq);
+                                                                 v.ghostsq);
     return cudaGetLastError();
 }
 
@@ -376,7 +373,7 @@ const KernelSet *kernel_set() {
 }
 
 // ------------------------------------------------------------------ tensor-product sets
-template <class L1, class T>
+template <class T>
 TPArgs<T> make_tp_args(const CtxView &v, const void *fin, void *fout) {
     TPArgs<T> a;
     a.fin = static_cast<const T *>(fin);
@@ -384,7 +381,6 @@ TPArgs<T> make_tp_args(const CtxView &v, const void *fin, void *fout) {
     a.inst = v.inst;
     a.tiles = v.tiles;
     a.ghosts = static_cast<const T *>(v.ghosts);
-    a.ghostsd = v.ghostsd;
     a.health = v.health;
     a.plane_idx = v.plane_idx;
     a.stride = v.stride;
@@ -468,7 +464,7 @@ cudaError_t tp_launch_block_w(const CtxView &v, const TPArgs<T> &a, const void *
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_step(const CtxView &v, const void *fin, void *fout) {
-    TPArgs<T> a = make_tp_args<L1, T>(v, fin, fout);
+    TPArgs<T> a = make_tp_args<T>(v, fin, fout);
     if (v.tile_width == 1) {  // one cell per block (D1Q9-P1 sets only: its tables fit in 48 KB)
         if constexpr (L1::Q1 == 9) {
             if constexpr (std::is_same<T, double>::value) {
@@ -499,7 +495,7 @@ cudaError_t tp_launch_step(const CtxView &v, const void *fin, void *fout) {
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_moments(const CtxView &v, const void *f, double *out, unsigned mask) {
-    const TPArgs<T> a = make_tp_args<L1, T>(v, f, nullptr);
+    const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
     // small double problems: one block per cell, as the step
     if constexpr (L1::Q1 == 9 && std::is_same<T, double>::value)
         if (v.ncells <= 48ll * v.num_sms) {
@@ -515,16 +511,16 @@ cudaError_t tp_launch_moments(const CtxView &v, const void *f, double *out, unsi
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_fill(const CtxView &v, void *f, const double *rho, const double *u, const double *theta) {
-    const TPArgs<T> a = make_tp_args<L1, T>(v, nullptr, f);
+    const TPArgs<T> a = make_tp_args<T>(v, nullptr, f);
     tp_fill_kernel<L1, N, T><<<v.ntiles, 32, 0, v.stream>>>(a, rho, u, theta, v.ncells);
     return cudaGetLastError();
 }
 
 template <class L1, int N, class T>
-cudaError_t tp_launch_ghost(const CtxView &v, const double *states, int ninst, void *ghosts, double *ghostsd) {
-    const TPArgs<T> a = make_tp_args<L1, T>(v, nullptr, nullptr);
+cudaError_t tp_launch_ghost(const CtxView &v, const double *states, int ninst, void *ghosts) {
+    const TPArgs<T> a = make_tp_args<T>(v, nullptr, nullptr);
     const int n = 2 * ninst;
-    tp_ghost_kernel<L1, N, T><<<(n + 63) / 64, 64, 0, v.stream>>>(a, states, ninst, static_cast<T *>(ghosts), ghostsd);
+    tp_ghost_kernel<L1, N, T><<<(n + 63) / 64, 64, 0, v.stream>>>(a, states, ninst, static_cast<T *>(ghosts));
     return cudaGetLastError();
 }
 
@@ -576,7 +572,7 @@ cudaError_t tp_persist_block_w(const CtxView &v, const TPArgs<T> &a, void *fa, v
 // occ non-null: report the resident blocks per SM instead of launching
 template <class L1, int N, class T>
 cudaError_t tp_persist_dispatch(const CtxView &v, void *fa, void *fb, int nsteps, int grid, int *occ) {
-    const TPArgs<T> a = make_tp_args<L1, T>(v, fa, fb);
+    const TPArgs<T> a = make_tp_args<T>(v, fa, fb);
     if constexpr (std::is_same<T, float>::value)
         if (v.fixedx && v.tensor_cores)
             return v.plane_identity ? tp_persist_block_w<L1, N, T, true, true, true>(v, a, fa, fb, nsteps, grid, occ)
@@ -708,7 +704,7 @@ namespace smrt {
 template <class L1, int N, class T>
 cudaError_t tp_launch_adj_step(const CtxView &v, const void *f, const double *lam_next, double *lam_t,
                                double *partials, double *dtau) {
-    const TPArgs<T> a = make_tp_args<L1, T>(v, f, nullptr);
+    const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
     if (v.fixedx)
         tp_adjoint_step_kernel<L1, N, T, true><<<v.ntiles, 32, 0, v.stream>>>(a, lam_next, lam_t, partials);
     else
@@ -721,7 +717,7 @@ cudaError_t tp_launch_adj_step(const CtxView &v, const void *f, const double *la
 
 template <class L1, int N, class T>
 cudaError_t tp_launch_adj_moments(const CtxView &v, const void *f, const double *gbar, unsigned mask, double *lam) {
-    const TPArgs<T> a = make_tp_args<L1, T>(v, f, nullptr);
+    const TPArgs<T> a = make_tp_args<T>(v, f, nullptr);
     if (v.fixedx)
         tp_adjoint_moments_kernel<L1, N, T, true><<<v.ntiles, 32, 0, v.stream>>>(a, gbar, mask, lam, v.ncells);
     else

@@ -64,16 +64,15 @@ struct StepArgs {
     const InstanceInfo *__restrict__ inst;
     const int2 *__restrict__ tiles;  // line kernel: (instance, first x) per block
     const T *__restrict__ ghosts;    // [instance][2][Q], library order
-    const double *__restrict__ ghostsd;  // the same end-state deviations in double
-    const long long *__restrict__ ghostsq;  // ... and in fixed point (split precision)
+    const long long *__restrict__ ghostsq;  // the same in fixed point (split precision)
     unsigned *health;
+    double cd;                // c in double
     long long plane[Lat::Q];  // element offset of each population plane, library order
     T wp[Lat::NP + 1];        // weight of the rest velocity, then of each pair
     double wpd[Lat::NP + 1];  // the same weights in double, for every double-precision rebuild
     float wsh[Lat::NP + 1];   // w 2^(24 - kFixP) as two-float numbers (split precision)
     float wsl[Lat::NP + 1];
     T c;
-    double cd;                // c in double
     float clo;                // c - float(c)
     int nx, ny, nz;           // box kernel geometry
     int kx, ky, kz;           // box kernel frame shift
@@ -379,14 +378,9 @@ struct Collide {
     // the constant a^gamma per monomial that does not vanish on the orbit.
     template <int Nm, class U>
     SMRT_D static void raw_moments(const U (&f)[Q], U (&R)[nmom(Nm)]) {
-        raw_moments_of<Nm>([&](auto I) { return f[decltype(I)::value]; }, R);
-    }
-    // ... with population i read as get(ic<i>) where it is needed (a pull, for the split step)
-    template <int Nm, class U, class Get>
-    SMRT_D static void raw_moments_of(Get &&get, U (&R)[nmom(Nm)]) {
         constexpr int Mm = nmom(Nm);
         static_for<Mm>([&](auto G) { R[decltype(G)::value] = U(0); });
-        R[0] = get(ic<0>{});
+        R[0] = f[0];
         static_for<kOrb.n>([&](auto O) {
             constexpr int o = decltype(O)::value;
             constexpr int np = 1 << (kOrb.k[o] - 1);
@@ -394,7 +388,7 @@ struct Collide {
             static_for<np>([&](auto B) {
                 constexpr int b = decltype(B)::value, p = kOrb.pair[o][b];
                 constexpr bool fl = kOrb.flip[o][b] != 0;
-                const U fp = get(ic<2 * p + 1>{}), fm = get(ic<2 * p + 2>{});
+                const U fp = f[2 * p + 1], fm = f[2 * p + 2];
                 S[b] = fp + fm;
                 D[b] = fl ? fm - fp : fp - fm;
             });
@@ -1045,7 +1039,7 @@ SMRT_D void line_tile(const StepArgs<Lat, T> &a, const T *__restrict__ fin, T *_
     };
     bool ok;
     if constexpr (Split) {
-        // ... in fixed point (the exact double end state beyond a fixed end)
+        // ... in fixed point (the end states are, from double values)
         float probe = 0.f;  // NaN once a non-finite value has been pulled
         ok = C::collide_split(
             [&](int i, const signed char *e, int s, int) -> long long {
@@ -1151,7 +1145,7 @@ __global__ void __launch_bounds__(128, kStepMinBlocks<Split>) step_line_persiste
 // order), rounded out to 16 bytes, brings all Q rows in by one copy, completion counted in
 // bytes on the warp's mbarrier. The lanes then read their pulls from shared memory instead of
 // issuing Q dependent loads each. Pulls from beyond a fixed end read the end states (in
-// double, exactly) and wrapped pulls of a periodic line read the state directly.
+// fixed point) and the edge warps of a periodic line read the state directly.
 template <class Lat>
 struct LineStage {
     static constexpr int kEmax = x_reach<Lat>();
@@ -1464,7 +1458,7 @@ __global__ void __launch_bounds__(128) fill_kernel(StepArgs<Lat, T> a, const dou
 // End-state populations of instance j: states[j] = (rho, u_phys, theta) left then right.
 template <class Lat, int N, class T>
 __global__ void ghost_kernel(StepArgs<Lat, T> a, const double *states, int ninst, T *ghosts,
-                             double *ghostsd, long long *ghostsq) {
+                             long long *ghostsq) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 2 * ninst) return;
     const int j = t / 2;
@@ -1476,7 +1470,6 @@ __global__ void ghost_kernel(StepArgs<Lat, T> a, const double *states, int ninst
     static_for<Lat::Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         ghosts[(long long)t * Lat::Q + i] = T(out[i]);
-        ghostsd[(long long)t * Lat::Q + i] = out[i];
         ghostsq[(long long)t * Lat::Q + i] = to_fixed(out[i]);
     });
 }

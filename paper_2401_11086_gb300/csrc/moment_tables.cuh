@@ -20,11 +20,6 @@ struct SlotIndex {
             ord[p] = c[p][0] + c[p][1] + c[p][2];
         }
     }
-    constexpr int with(int p, int k, int v) const {
-        int e[3] = {c[p][0], c[p][1], c[p][2]};
-        e[k] = v;
-        return mi_pos(e[0], e[1], e[2]);
-    }
 };
 
 constexpr double fact_small(int n) {

@@ -75,12 +75,11 @@ struct TPArgs {
     const InstanceInfo *__restrict__ inst;
     const int2 *__restrict__ tiles;    // (instance, first x) per block
     const T *__restrict__ ghosts;      // [instance][2][Q], library order
-    const double *__restrict__ ghostsd;
     unsigned *health;
     const int *__restrict__ plane_idx; // caller plane of each library population
     long long stride;                  // elements per population plane
-    double w1[kMaxQ1];                 // 1D weights, library order
     double cd;                         // lattice scale c
+    double w1[kMaxQ1];                 // 1D weights, library order
     unsigned step;
     int tma;                           // 1: the kernel's tensor maps describe fin and fout
     int ident;                         // 1: library population i is caller plane i
@@ -1204,19 +1203,19 @@ struct TPCellGroup {
     int lane;
     SMRT_D void sync() const { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 };
-template <class L1, int N, bool Adjoint>
+template <class L1, int N>
 struct TPLaneShared {
     static constexpr int Q1 = L1::Q1, P2 = Q1 * Q1, Q = P2 * Q1, M = nmom(N);
     static constexpr int kJK = (N + 1) * (N + 2) / 2;  // (j, k) with j + k <= N
     using C = LaneCell<N>;
     LaneMoments<N> m;
-    double f[(Q + 1) / 2 * 2];      // populations, library order (the adjoint: then lam's)
+    double f[(Q + 1) / 2 * 2];      // populations, library order
     double g[P2][N + 1];            // x-row sums g_j of row b + d c; x-row coefficients of the rebuild
     double pw[Q1][N + 1];           // e_a^j
     double w[Q1 + 1];
     double h[Q1][kJK];              // per z-plane c: sums over y; plane coefficients of the rebuild
     double cp[N + 1 + (N & 1 ? 0 : 1)];
-    double V[Adjoint ? int(C::kAdjoint) : int(C::kForward)];
+    double V[C::kForward];
     // (j, k) of index r, j ascending then k, three bits each
     SMRT_HD static constexpr unsigned long long packed(bool second) {
         unsigned long long v = 0;
@@ -1309,8 +1308,7 @@ struct TPLaneShared {
         }
     }
     // tables of the block (no barrier)
-    template <class T>
-    SMRT_D void load(const TPArgs<T> &a) {
+    SMRT_D void load(const TPArgs<double> &a) {
         lane_copy(m, lane_moments<N>());
         if (threadIdx.x < Q1) {
             const double ea = e1<L1>(threadIdx.x);
@@ -1323,14 +1321,14 @@ struct TPLaneShared {
         }
     }
     // the cell's pulled populations and the tables, all in flight together (no barrier)
-    template <bool FixedX, class T, class Plane>
-    SMRT_D void pull(const TPArgs<T> &a, const T *gl, int x, int L, int kx, Plane &&plane) {
+    template <bool FixedX, class Plane>
+    SMRT_D void pull(const TPArgs<double> &a, const double *gl, int x, int L, int kx, Plane &&plane) {
         constexpr int kPer = (Q + 127) / 128;
-        T v[kPer];
+        double v[kPer];
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
             const int i = threadIdx.x + 128 * r;
-            v[r] = T(0);
+            v[r] = 0.0;
             if (i < Q) {
                 const int t = x - e1<L1>(i % Q1) - kx;
                 if (FixedX && t < 0)
@@ -1344,14 +1342,14 @@ struct TPLaneShared {
         load(a);
 #pragma unroll
         for (int r = 0; r < kPer; ++r)
-            if (threadIdx.x + 128 * r < Q) f[threadIdx.x + 128 * r] = double(v[r]);
+            if (threadIdx.x + 128 * r < Q) f[threadIdx.x + 128 * r] = v[r];
     }
     SMRT_D double weight(int i) const { return w[i % Q1] * w[i / Q1 % Q1] * w[i / P2]; }
 };
 
 template <class L1, int N, bool FixedX>
 __global__ void __launch_bounds__(128) tp_step_cell_lanes(TPArgs<double> a) {
-    using SH = TPLaneShared<L1, N, false>;
+    using SH = TPLaneShared<L1, N>;
     constexpr int Q1 = SH::Q1, Q = SH::Q;
     __shared__ __align__(16) unsigned char raw[sizeof(SH)];
     SH &s = *reinterpret_cast<SH *>(raw);
@@ -1383,7 +1381,7 @@ __global__ void __launch_bounds__(128) tp_step_cell_lanes(TPArgs<double> a) {
 // 208 -> 20 us, one thread per cell being 4 warps on the whole GPU.
 template <class L1, int N, bool FixedX>
 __global__ void __launch_bounds__(128) tp_moments_cell_lanes(TPArgs<double> a, double *out, long long ncells, unsigned mask) {
-    using SH = TPLaneShared<L1, N, false>;
+    using SH = TPLaneShared<L1, N>;
     using C = LaneCell<N>;
     __shared__ __align__(16) unsigned char raw[sizeof(SH)];
     SH &s = *reinterpret_cast<SH *>(raw);
@@ -1488,8 +1486,7 @@ __global__ void __launch_bounds__(128) tp_fill_kernel(TPArgs<T> a, const double 
 
 // End-state populations of every instance, library order: thread t = 2 j + side.
 template <class L1, int N, class T>
-__global__ void __launch_bounds__(64) tp_ghost_kernel(TPArgs<T> a, const double *states, int ninst, T *ghosts,
-                                                      double *ghostsd) {
+__global__ void __launch_bounds__(64) tp_ghost_kernel(TPArgs<T> a, const double *states, int ninst, T *ghosts) {
     __shared__ TPTables<L1, double> s;
     tp_load_tables<L1>(a, s);
     using C = TPCell<L1, N, double>;
@@ -1502,11 +1499,7 @@ __global__ void __launch_bounds__(64) tp_ghost_kernel(TPArgs<T> a, const double 
     double P[C::M];
     C::template equilibrium<double>(st[0], uu, st[4], a.cd, P);
     T *g = ghosts + (long long)t * Q;
-    double *gd = ghostsd + (long long)t * Q;
-    C::template rebuild<double>(P, s.e, s.w, [&](int i, double v) {
-        g[i] = T(v);
-        gd[i] = v;
-    });
+    C::template rebuild<double>(P, s.e, s.w, [&](int i, double v) { g[i] = T(v); });
 }
 
 }  // namespace smrt
