@@ -365,8 +365,6 @@ def run_batched(args, world: int, rank: int, local: int) -> None:
     value = rate / 1e9
     peak, peak_kind = measured_peak()
     achieved = 2.0 * q * 4 * cells * K / (ms * 1e-3) / 1e9
-    # the FP64 pipe bounds this kernel: its double-precision operations per cell-step (ncu
-    # instruction counts, an FMA counted as two) against the nominal FP64 rate
     # the kernel is bound by instruction issue (ncu: 47 % issue-active, instruction-fetch stalls
     # first): its warp instructions per cell-step against one per clock per scheduler
     ginst = BATCHED_WARP_INST_PER_CELL * cells * K / (ms * 1e-3) / 1e9
@@ -400,7 +398,7 @@ def run_batched(args, world: int, rank: int, local: int) -> None:
 # double-precision operations per cell-step of the D3Q729, N = 5 step kernel (ncu: DFMA x 2 +
 # DADD + DMUL over one launch of the 512-shock workload, divided by its cells), and the
 # nominal FP64 rate of a GB300
-TP_FP64_FLOP_PER_CELL = 14949.0
+TP_FP64_FLOP_PER_CELL = 13216.0
 FP64_PEAK_GFLOPS = 1250.0
 # warp instructions per cell-step of the split-precision D3Q103, N = 4 staged line kernel on the
 # 64 batched shocks (ncu smsp__inst_executed.sum of one plain launch / cells), and the issue rate of a GB300 (4 schedulers per SM,

@@ -272,10 +272,11 @@ lb_status lb_moments(lb_ctx *ctx, const void *f, double *out, unsigned which_mas
  * times tau_c,nm. Arithmetic is double whatever the precision of f_t. Populations pulled from
  * beyond a fixed x end are constants (no gradient). The per-block gradient partials live in a
  * scratch array owned by the context; calls on one context must not overlap.
- * Every set has adjoint kernels; on D3Q729 and D3Q4913 the projection of lam_next and the
- * evaluation of the raw moments' adjoint factor over the axes as the forward step does (D3Q39
- * and D3Q103 lines of at most 32 cells per SM take a group of 16 or 32 threads per cell,
- * otherwise one thread per cell, 32-cell tiles, the per-tile gradient partials reduced in tile order).
+ * Every set has adjoint kernels: a group of 16 or 32 threads per cell for D3Q39 and D3Q103 lines
+ * of at most 32 cells per SM, one thread per cell on every other grid. On D3Q729 and D3Q4913 the
+ * projection of lam_next and the evaluation of the raw moments' adjoint factor over the axes as
+ * the forward step does. The gradient partials are summed within a block and then over the blocks
+ * in fixed orders: dtau does not depend on scheduling.
  * Errors: LB_ERR_INVALID (null, lam_next overlapping lam_t, relaxation unset), LB_ERR_UNSUPPORTED
  * (an instance using the ES-BGK model), LB_ERR_CUDA. */
 lb_status lb_step_adjoint(lb_ctx *ctx, const void *f_t, const double *lam_next, double *lam_t,

@@ -11,8 +11,8 @@
 // weights). Between them sits the moment-space VJP shared with the other sets (moment_vjp in
 // adjoint.cuh). One thread per cell, 32-cell tiles; the streaming transpose is the push of
 // adjoint_kernels.cuh (every lam^t_i(y) written once, zero where nothing pulls from y); the
-// relaxation-time gradients are reduced per tile by a warp shuffle in a fixed order, then over
-// tiles in tile order.
+// relaxation-time gradients are reduced per tile by a warp shuffle, then over the tiles by
+// reduce_partials_kernel, both in a fixed order.
 #pragma once
 
 #include "adjoint.cuh"
