@@ -58,6 +58,7 @@ struct lb_ctx {
     int2 *d_btiles;      // tensor-product lines: block tiles of the step kernels (tile_width cells)
     int *d_plane;        // tensor-product sets: caller plane of each library population
     void *d_ghosts;
+    double *d_ghostsd;     // D3Q39 / D3Q103: the end states in double
     long long *d_ghostsq;  // D3Q39 / D3Q103: the end states in fixed point
     double *d_states;
     unsigned *d_health;  // [0] health flags, [1..3] grid barrier and step counter
@@ -190,6 +191,7 @@ void free_tables(lb_ctx *c) {
     cudaFree(c->d_ltiles);
     cudaFree(c->d_plane);
     cudaFree(c->d_ghosts);
+    cudaFree(c->d_ghostsd);
     cudaFree(c->d_ghostsq);
     cudaFree(c->d_states);
     cudaFree(c->d_health);
@@ -364,6 +366,7 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
     if (e == cudaSuccess && line && tensor) e = cudaMalloc(&c->d_btiles, sizeof(int2) * c->max_tiles);
     if (e == cudaSuccess && tensor) e = cudaMalloc(&c->d_plane, sizeof(int) * c->q);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_ghosts, c->elem * c->q * 2 * grid->batch);
+    if (e == cudaSuccess && !tensor) e = cudaMalloc(&c->d_ghostsd, sizeof(double) * c->q * 2 * grid->batch);
     if (e == cudaSuccess && !tensor) e = cudaMalloc(&c->d_ghostsq, sizeof(long long) * c->q * 2 * grid->batch);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_states, sizeof(double) * 10 * grid->batch);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_health, 16);
@@ -439,6 +442,7 @@ extern "C" lb_status lb_init_lattice(lb_ctx **out, const lb_lattice_desc *lat, c
     v.ltiles = c->d_ltiles;
     v.plane_idx = c->d_plane;
     v.ghosts = c->d_ghosts;
+    v.ghostsd = c->d_ghostsd;
     v.ghostsq = c->d_ghostsq;
     v.health = c->d_health;
     v.bar = c->d_health + 1;
@@ -469,7 +473,10 @@ lb_status flush_tables(lb_ctx *c) {
             // a view whose instance table starts at j0
             CtxView gv = c->view;
             gv.inst = c->d_inst + j0;
-            if (c->d_ghostsq) gv.ghostsq = c->d_ghostsq + (size_t)c->q * 2 * j0;
+            if (c->d_ghostsq) {
+                gv.ghostsd = c->d_ghostsd + (size_t)c->q * 2 * j0;
+                gv.ghostsq = c->d_ghostsq + (size_t)c->q * 2 * j0;
+            }
             e = c->ks->ghost(gv, c->d_states + 10 * (size_t)j0, j1 - j0,
                              static_cast<char *>(c->d_ghosts) + c->elem * c->q * 2 * (size_t)j0);
         }

@@ -32,7 +32,8 @@ struct CtxView {
     const int2 *tiles;
     int ntiles;
     const void *ghosts;
-    long long *ghostsq;  // the end states in fixed point (D3Q39, D3Q103)
+    double *ghostsd;     // the end states in double and
+    long long *ghostsq;  // in fixed point (D3Q39, D3Q103)
     unsigned *health;
     long long ncells;
     unsigned step;   // launch counter of lb_step (seeds the stochastic rounding)
@@ -84,6 +85,7 @@ StepArgs<Lat, T> make_args(const CtxView &v, const void *fin, void *fout) {
     a.inst = v.inst;
     a.tiles = v.tiles;
     a.ghosts = static_cast<const T *>(v.ghosts);
+    a.ghostsd = v.ghostsd;
     a.ghostsq = v.ghostsq;
     a.health = v.health;
     for (int i = 0; i < Lat::Q; ++i) a.plane[i] = v.plane[i];
@@ -289,7 +291,7 @@ cudaError_t launch_ghost(const CtxView &v, const double *states, int ninst, void
     const StepArgs<Lat, T> a = make_args<Lat, T>(v, nullptr, nullptr);
     const int n = 2 * ninst;
     ghost_kernel<Lat, N, T><<<(n + 63) / 64, 64, 0, v.stream>>>(a, states, ninst, static_cast<T *>(ghosts),
-                                                                 v.ghostsq);
+                                                                 v.ghostsd, v.ghostsq);
     return cudaGetLastError();
 }
 
